@@ -212,7 +212,7 @@ typedef struct hg_grid_info {
     int32_t kind;
     int32_t max_depth;      /* deepest node in the node list (k-d splits or octree levels) */
     int64_t n_nodes, n_leaves;
-    int64_t n_tail;         /* stored neighbor entries beyond each wall's first */
+    int64_t n_tail;         /* stored neighbor entries beyond each wall's first (96-byte records; else 1) */
     int64_t device_bytes;   /* HBM held by the grid */
     int64_t long_walls;     /* walls whose list is longer than the scan limit (searched top-down from the
                                wall's rope node, the deepest node across the wall covering it) */
@@ -226,9 +226,16 @@ typedef struct hg_grid_info {
 
 /* Upload a grid: the node list of Sect. 2.2 and the six per-leaf neighbor
  * lists of Sect. 2.3 (built once with the grid, sorted by decreasing overlap
- * area) become 96-byte leaf records holding each wall's list head, the list
- * tails and the descent nodes of the top-down search (Sect. 2.3), in device
- * memory owned by the returned handle until hg_free_grid.  desc and the
+ * area) become leaf records and the descent nodes of the top-down search
+ * (Sect. 2.3), in device memory owned by the returned handle until
+ * hg_free_grid.  When every bound is a single-precision number (0, or of
+ * magnitude 2^-60 to 2^20, the largest at least 2^-20; every dyadic tree of
+ * a domain such as [-1, 1]^3 down to level 23) a record is 64 bytes: the
+ * bounds in single precision, without loss, and per wall the one neighbor,
+ * the first of two or four equal neighbors with their id steps, or the node
+ * covering the wall (see hg_build_ropes) for other lists.  Otherwise it is 96
+ * bytes with each wall's list head, and the list tails follow.  Results do
+ * not depend on the record.  desc and the
  * arrays it points to are host memory, read during the call only.  With
  * validate != 0 the description is checked first
  * (links in range, children tiling their parent, leaf ids, every neighbor
@@ -295,18 +302,21 @@ hg_status hg_load_grid_ropes(const hg_grid_desc *desc, const int32_t *ropes, int
 typedef struct hg_trace_opts {
     int32_t precision;   /* HG_FP64 or HG_FP32K */
     int32_t block;       /* threads per block (32..256, multiple of 32); 0 = tuned or default */
-    int32_t smem_nodes;  /* top tree nodes the walks stage in shared memory (clamped to 200 KB); -1 = tuned or
-                            default (64: the walk descends only after edge and corner exits and list misses, and
-                            shared memory is taken from the L1 that serves its record gathers).  The setup pass
+    int32_t smem_nodes;  /* top tree nodes the walks of 96-byte records stage in shared memory (clamped to 200 KB);
+                            -1 = tuned or default (64: the walk descends only after edge and corner exits and list
+                            misses, and shared memory is taken from the L1 that serves its record gathers).  Walks
+                            of 64-byte records stage none (accepted and checked, then ignored).  The setup pass
                             (first leaf of every ray) always stages the top 8 KB */
     int32_t schedule;    /* 0 = tuned or automatic; 1 = static ray stride; 2 = dynamic queue (warp-aggregated
                             counter) in input order; 3 = dynamic queue, rays with the most estimated
                             crossings first (automatic when there are fewer than 48 rays per
                             resident thread) */
     int32_t min_blocks;  /* 0 = tuned or default (4; 3 for hg_find_interactions, whose walk needs more
-                            than 64 registers); 3 or 4 resident 256-thread blocks per SM the kernel's
-                            register budget is cut for (80 or 64 registers; each walking thread also keeps
-                            its ray's origin, direction and 1/d in 72 bytes of shared memory) */
+                            than 64 registers); 3 or 4 resident 256-thread blocks per SM the register
+                            budget of the walks of 96-byte records is cut for (80 or 64 registers; each walking
+                            thread also keeps its ray's origin, direction and 1/d in 72 bytes of shared
+                            memory).  Walks of 64-byte records have one form of 64 registers (accepted and
+                            checked, then ignored) */
     int32_t split;       /* HG_SPLIT_AUTO (0), HG_SPLIT_OFF or HG_SPLIT_FORCE; see below */
     int64_t max_steps;   /* per-ray step limit; 0 = 4 * n_leaves + 64 */
 } hg_trace_opts;
@@ -351,12 +361,12 @@ hg_status hg_trace_rays_rho(const hg_grid *g, int64_t n, const double *o, const 
  * additions where hg_trace_rays cuts a long path into segments (a few ulps).
  * It walks every path whole, each thread taking rays at a static stride,
  * whatever opts.schedule and opts.split ask for (they are accepted and
- * checked, then ignored).  Its scratch -- one 48-byte start record per ray
+ * checked, then ignored).  Its scratch -- one start record of at most 64 bytes per ray
  * and a work counter -- comes from a fixed array compiled into the library;
  * it calls no cudaMalloc, cudaFree or other allocator.
  *   - n must not exceed HG_NOALLOC_MAX_RAYS; a larger n returns HG_EINVAL
  *     before anything is launched (split the batch, or use hg_trace_rays).
- *   - Every GPU that loads the library holds the array (about 12.6 MB)
+ *   - Every GPU that loads the library holds the array (about 16.8 MB)
  *     until the process exits.
  *   - The first call on a device looks the array's device address up
  *     (cudaGetSymbolAddress) with that device current; make that first call
@@ -519,8 +529,9 @@ hg_status hg_sum_i32(int64_t n, const int32_t *x, int64_t *out, hg_stream stream
  * batched form is this library's own: the optical-depth pass of
  * hg_trace_rays (same contract and results, whole paths, never split) over
  * many grids of uneven size, each with its own ray range, traced in one
- * persistent launch: ray chunks of every grid form one work list that
- * resident blocks drain through an atomic counter, larger grids first.
+ * persistent launch (two when grids of 64-byte and of 96-byte records are
+ * mixed): ray chunks of every grid form one work list that resident blocks
+ * drain through an atomic counter, larger grids first.
  * ray_begin (host i64[n_grids+1]) splits the concatenated ray and output
  * arrays by grid.  The batch holds a device table of the grids (which
  * must outlive it) and a reusable work counter; hg_batch_trace may be

@@ -25,6 +25,7 @@ ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 # (source, needs -fmad=false)
 UNITS = [
     ("trace.cu", True),
+    ("tracef.cu", True),
     ("batch.cu", True),
     ("noalloc.cu", True),
     ("gbuild.cu", True),

@@ -14,7 +14,8 @@
 #include <vector>
 
 #include "hg_internal.h"
-#include "walk.cuh"
+#include "trace_args.cuh"
+#include "walkf.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -45,7 +46,7 @@ struct BatchArgs {
     uint8_t *status;
     int64_t max_steps;  // 0: per grid 4 n_leaves + 64
     unsigned long long *counter;
-    RayStart *starts;   // [total] start records, indexed by ray
+    void *starts;       // [total] start records (RayStart or RayStartF), indexed by ray
 };
 
 // Queue position -> slot (grid in processing order) by binary search.
@@ -61,7 +62,9 @@ __device__ __forceinline__ int queue_slot(const int64_t *s_qbeg, int n_grids, in
     return lo;
 }
 
-// Setup pass over the whole batch (checks, 1/d, clip, first leaf).
+// Setup pass over the whole batch (checks, 1/d, clip, first leaf).  F: the grids hold single-precision
+// records.
+template <bool F>
 __global__ void __launch_bounds__(256) batch_setup_kernel(const BatchArgs A) {
     __shared__ int64_t s_qbeg[kMaxBatch + 1];
     __shared__ int32_t s_perm[kMaxBatch];
@@ -72,7 +75,17 @@ __global__ void __launch_bounds__(256) batch_setup_kernel(const BatchArgs A) {
         const int slot = queue_slot(s_qbeg, A.n_grids, q);
         const BatchEntry *E = A.E + s_perm[slot];
         const int64_t ray = E->ray0 + (q - s_qbeg[slot]);
-        A.starts[ray] = ray_setup<2>(E->G, nullptr, 0, A.o, A.d, A.smax, ray);
+        const DevGrid &G = E->G;
+        const RayStart R = ray_setup(
+            G,
+            [&](long long p0, long long p1, long long p2, uint32_t sg) {
+                return F ? locate_key_f<2>(G, nullptr, 0, p0, p1, p2, sg) : descend<2>(G, nullptr, 0, p0, p1, p2, sg);
+            },
+            A.o, A.d, A.smax, ray);
+        if (F)
+            static_cast<RayStartF *>(A.starts)[ray] = start_f(R, A.o, A.d, ray);
+        else
+            static_cast<RayStart *>(A.starts)[ray] = R;
     }
 }
 
@@ -98,14 +111,41 @@ struct BatchRays {
         ms = (int32_t)(m < 0x7fffffff ? m : 0x7fffffff);
         return true;
     }
+    // Up to 32 items for the calling warp (GridRays::grab); with each item's grid.
+    __device__ __forceinline__ int grab(PoolItem *pool, const WalkIO &) const {
+        const int lane = threadIdx.x & 31;
+        unsigned long long base = 0;
+        if (lane == 0) base = atomicAdd(A->counter, 32ULL);
+        base = __shfl_sync(0xffffffffu, base, 0);
+        const int64_t q = (int64_t)base + lane;
+        const bool ok = q < A->total;
+        if (ok) {
+            const int slot = queue_slot(s_qbeg, A->n_grids, q);
+            const int32_t g = s_perm[slot];
+            PoolItem P;
+            P.item = A->E[g].ray0 + (q - s_qbeg[slot]);
+            P.of = g;
+            pool[lane] = P;
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(static_cast<const RayStartF *>(A->starts) + P.item));
+        }
+        return __popc(__ballot_sync(0xffffffffu, ok));
+    }
+    __device__ __forceinline__ void item(const PoolItem &P, const DevGrid *&g, int32_t &ms) const {
+        const BatchEntry *E = A->E + P.of;
+        g = &E->G;
+        const int64_t m = A->max_steps > 0 ? A->max_steps : E->max_steps;
+        ms = (int32_t)(m < 0x7fffffff ? m : 0x7fffffff);
+    }
 };
 
-// NAV: 0 every grid holds neighbor lists, 1 every grid ropes, 2 a mix (read per grid).
+// NAV: 0 every grid holds neighbor lists, 1 every grid ropes, 2 a mix (read per grid); 3 the grids hold
+// single-precision records with either.
 template <int PREC, int NAV>
-__global__ void __launch_bounds__(256) batch_kernel(const BatchArgs A) {
+__global__ void __launch_bounds__(256, NAV == 3 ? 4 : 1) batch_kernel(const BatchArgs A) {
     __shared__ int64_t s_qbeg[kMaxBatch + 1];
     __shared__ int32_t s_perm[kMaxBatch];
-    __shared__ double s_geo[9 * 256];  // the walking threads' ray geometry (blocks of at most 256)
+    // the walking threads' ray geometry (blocks of at most 256)
+    __shared__ __align__(16) unsigned char s_geo[256 * (NAV == 3 ? kGeoBytesF : kGeoBytes)];
     for (int i = threadIdx.x; i <= A.n_grids; i += blockDim.x) s_qbeg[i] = A.qbeg[i];
     for (int i = threadIdx.x; i < A.n_grids; i += blockDim.x) s_perm[i] = A.perm[i];
     __syncthreads();
@@ -119,20 +159,30 @@ __global__ void __launch_bounds__(256) batch_kernel(const BatchArgs A) {
     io.tau = A.tau;
     io.ncross = A.ncross;
     io.status = A.status;
-    walk_loop<2, MODE_TAU, PREC, NAV>(src, io, nullptr, 0, s_geo);
+    if constexpr (NAV == 3) {
+        __shared__ PoolItem s_pool[256];
+        walk_loop_f<MODE_TAU, PREC>(src, io, s_geo, s_pool);
+    } else
+        walk_loop<2, MODE_TAU, PREC, NAV>(src, io, nullptr, 0, reinterpret_cast<double *>(s_geo));
 }
 
 }  // namespace hg
 
+// The grids of a batch in one or two queues, one launch each: those with double-precision records and those
+// with single-precision ones.
 struct hg_batch {
+    struct Queue {
+        int n_grids = 0;
+        int64_t total = 0;
+        int64_t *d_qbeg = nullptr;
+        int32_t *d_perm = nullptr;
+        unsigned long long *d_counter = nullptr;
+        int nav = 0;  // as batch_kernel's NAV
+    } q[2];
     int n_grids = 0;
-    int64_t total = 0;
+    int64_t total = 0;  // rays of the whole batch
     hg::BatchEntry *d_entries = nullptr;
-    int64_t *d_qbeg = nullptr;
-    int32_t *d_perm = nullptr;
-    unsigned long long *d_counter = nullptr;
     int device = 0;
-    int nav = 0;  // 0 all grids with neighbor lists, 1 all with ropes, 2 mixed
 };
 
 using namespace hg;
@@ -157,31 +207,39 @@ extern "C" hg_status hg_batch_create(int32_t n_grids, const hg_grid *const *grid
             return HG_EINVAL;
         }
         ent[i].G = grids[i]->d;
-        ent[i].G.nodes = grids[i]->d.nodes;
         ent[i].ray0 = ray_begin[i];
         ent[i].max_steps = 4 * grids[i]->d.n_leaves + 64;
         cnt[i] = ray_begin[i + 1] - ray_begin[i];
     }
-    // largest ray counts first, so that the long queues start early
-    std::vector<int32_t> perm((size_t)n_grids);
-    std::iota(perm.begin(), perm.end(), 0);
-    std::stable_sort(perm.begin(), perm.end(), [&](int32_t a, int32_t b) { return cnt[a] > cnt[b]; });
-    std::vector<int64_t> qbeg((size_t)n_grids + 1, 0);
-    for (int s = 0; s < n_grids; s++) qbeg[s + 1] = qbeg[s] + cnt[perm[s]];
     hg_batch *b = new hg_batch();
     b->n_grids = n_grids;
-    int n_ropes = 0;
-    for (int i = 0; i < n_grids; i++) n_ropes += grids[i]->d.nav == HG_NAV_ROPES ? 1 : 0;
-    b->nav = n_ropes == 0 ? 0 : (n_ropes == n_grids ? 1 : 2);
-    b->total = qbeg[n_grids];
+    b->total = ray_begin[n_grids];
     cudaGetDevice(&b->device);
     cudaError_t e = cudaMalloc(&b->d_entries, ent.size() * sizeof(BatchEntry));
-    if (e == cudaSuccess) e = cudaMalloc(&b->d_qbeg, qbeg.size() * sizeof(int64_t));
-    if (e == cudaSuccess) e = cudaMalloc(&b->d_perm, perm.size() * sizeof(int32_t));
-    if (e == cudaSuccess) e = cudaMalloc(&b->d_counter, sizeof(unsigned long long));
     if (e == cudaSuccess) e = cudaMemcpy(b->d_entries, ent.data(), ent.size() * sizeof(BatchEntry), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(b->d_qbeg, qbeg.data(), qbeg.size() * sizeof(int64_t), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(b->d_perm, perm.data(), perm.size() * sizeof(int32_t), cudaMemcpyHostToDevice);
+    for (int f = 0; f < 2 && e == cudaSuccess; f++) {
+        hg_batch::Queue &Q = b->q[f];
+        std::vector<int32_t> perm;
+        int n_ropes = 0;
+        for (int i = 0; i < n_grids; i++)
+            if ((grids[i]->d.recf != nullptr) == (f == 1)) {
+                perm.push_back(i);
+                n_ropes += grids[i]->d.nav == HG_NAV_ROPES ? 1 : 0;
+            }
+        if (perm.empty()) continue;
+        // largest ray counts first, so that the long queues start early
+        std::stable_sort(perm.begin(), perm.end(), [&](int32_t x, int32_t y) { return cnt[x] > cnt[y]; });
+        std::vector<int64_t> qbeg(perm.size() + 1, 0);
+        for (size_t s = 0; s < perm.size(); s++) qbeg[s + 1] = qbeg[s] + cnt[perm[s]];
+        Q.n_grids = (int)perm.size();
+        Q.nav = f == 1 ? 3 : (n_ropes == 0 ? 0 : (n_ropes == Q.n_grids ? 1 : 2));
+        Q.total = qbeg.back();
+        e = cudaMalloc(&Q.d_qbeg, qbeg.size() * sizeof(int64_t));
+        if (e == cudaSuccess) e = cudaMalloc(&Q.d_perm, perm.size() * sizeof(int32_t));
+        if (e == cudaSuccess) e = cudaMalloc(&Q.d_counter, sizeof(unsigned long long));
+        if (e == cudaSuccess) e = cudaMemcpy(Q.d_qbeg, qbeg.data(), qbeg.size() * sizeof(int64_t), cudaMemcpyHostToDevice);
+        if (e == cudaSuccess) e = cudaMemcpy(Q.d_perm, perm.data(), perm.size() * sizeof(int32_t), cudaMemcpyHostToDevice);
+    }
     if (e != cudaSuccess) {
         hg_batch_free(b);
         return cuda_err(e, "hg_batch_create");
@@ -193,9 +251,11 @@ extern "C" hg_status hg_batch_create(int32_t n_grids, const hg_grid *const *grid
 extern "C" void hg_batch_free(hg_batch *b) {
     if (!b) return;
     cudaFree(b->d_entries);
-    cudaFree(b->d_qbeg);
-    cudaFree(b->d_perm);
-    cudaFree(b->d_counter);
+    for (auto &Q : b->q) {
+        cudaFree(Q.d_qbeg);
+        cudaFree(Q.d_perm);
+        cudaFree(Q.d_counter);
+    }
     delete b;
 }
 
@@ -215,10 +275,6 @@ extern "C" hg_status hg_batch_trace(hg_batch *b, const double *o, const double *
     cudaStream_t s = (cudaStream_t)stream;
     BatchArgs A{};
     A.E = b->d_entries;
-    A.qbeg = b->d_qbeg;
-    A.perm = b->d_perm;
-    A.n_grids = b->n_grids;
-    A.total = b->total;
     A.o = o;
     A.d = d;
     A.smax = s_max;
@@ -227,36 +283,48 @@ extern "C" hg_status hg_batch_trace(hg_batch *b, const double *o, const double *
     A.ncross = ncross;
     A.status = ray_status;
     A.max_steps = opts ? opts->max_steps : 0;
-    A.counter = b->d_counter;
     const int block = (opts && opts->block > 0) ? opts->block : 256;
     if (block < 32 || block > 256 || block % 32) {
         set_error("hg_batch_trace: block must be a multiple of 32 in 32..256");
         return HG_EINVAL;
     }
     using BatchFn = void (*)(const BatchArgs);
-    static const BatchFn kernels[2][3] = {{&batch_kernel<HG_FP64, 0>, &batch_kernel<HG_FP64, 1>, &batch_kernel<HG_FP64, 2>},
+    static const BatchFn kernels[2][4] = {{&batch_kernel<HG_FP64, 0>, &batch_kernel<HG_FP64, 1>, &batch_kernel<HG_FP64, 2>,
+                                           &batch_kernel<HG_FP64, 3>},
                                           {&batch_kernel<HG_FP32K, 0>, &batch_kernel<HG_FP32K, 1>,
-                                           &batch_kernel<HG_FP32K, 2>}};
-    const BatchFn kern = kernels[prec == HG_FP64 ? 0 : 1][b->nav];
-    int per_sm = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, block, 0);
-    if (e != cudaSuccess) return cuda_err(e, "batch occupancy");
-    int64_t blocks = (int64_t)std::max(1, per_sm) * sm_count();
-    blocks = std::min<int64_t>(blocks, (b->total + block - 1) / block);
-    RayStart *starts = nullptr;
-    e = cudaMallocAsync((void **)&starts, (size_t)b->total * sizeof(RayStart), s);
+                                           &batch_kernel<HG_FP32K, 2>, &batch_kernel<HG_FP32K, 3>}};
+    // start records of either kind, indexed by ray: two queues never share a record's bytes
+    const size_t rec = b->q[1].total > 0 ? sizeof(RayStartF) : sizeof(RayStart);
+    const size_t both = b->q[0].total > 0 && b->q[1].total > 0 ? (size_t)b->total * sizeof(RayStart) : 0;
+    unsigned char *starts = nullptr;
+    cudaError_t e = cudaMallocAsync((void **)&starts, (size_t)b->total * rec + both, s);
     if (e != cudaSuccess) return cuda_err(e, "batch start scratch");
-    A.starts = starts;
-    e = cudaMemsetAsync(b->d_counter, 0, sizeof(unsigned long long), s);
-    if (e != cudaSuccess) {
-        cudaFreeAsync(starts, s);
-        return cuda_err(e, "batch counter reset");
+    for (int f = 0; f < 2 && e == cudaSuccess; f++) {
+        const hg_batch::Queue &Q = b->q[f];
+        if (Q.total == 0) continue;
+        A.qbeg = Q.d_qbeg;
+        A.perm = Q.d_perm;
+        A.n_grids = Q.n_grids;
+        A.total = Q.total;
+        A.counter = Q.d_counter;
+        A.starts = f == 0 && both ? starts + (size_t)b->total * rec : starts;
+        const BatchFn kern = kernels[prec == HG_FP64 ? 0 : 1][Q.nav];
+        int per_sm = 0;
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, block, 0);
+        if (e != cudaSuccess) break;
+        int64_t blocks = (int64_t)std::max(1, per_sm) * sm_count();
+        blocks = std::min<int64_t>(blocks, (Q.total + block - 1) / block);
+        e = cudaMemsetAsync(Q.d_counter, 0, sizeof(unsigned long long), s);
+        if (e != cudaSuccess) break;
+        const int64_t sblocks = std::min<int64_t>((Q.total + 255) / 256, (int64_t)sm_count() * 8);
+        if (f == 1)
+            batch_setup_kernel<true><<<(unsigned)sblocks, 256, 0, s>>>(A);
+        else
+            batch_setup_kernel<false><<<(unsigned)sblocks, 256, 0, s>>>(A);
+        kern<<<(unsigned)blocks, block, 0, s>>>(A);
+        note_launches(2);
+        e = cudaGetLastError();
     }
-    const int64_t sblocks = std::min<int64_t>((b->total + 255) / 256, (int64_t)sm_count() * 8);
-    batch_setup_kernel<<<(unsigned)sblocks, 256, 0, s>>>(A);
-    kern<<<(unsigned)blocks, block, 0, s>>>(A);
-    note_launches(2);
-    e = cudaGetLastError();
     cudaFreeAsync(starts, s);
     return e == cudaSuccess ? HG_OK : cuda_err(e, "batch launch");
 }
@@ -278,7 +346,7 @@ extern "C" hg_status hg_autotune(hg_grid *g, int64_t n, const double *o, const d
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
-    const int node_bytes = g->d.kind == HG_KDTREE ? 16 : 32;
+    const int node_bytes = node_bytes_of(g->d);
     const int blocks[] = {128, 256};
     const int smem_kb[] = {0, 8, 32, 64};
     hg_trace_opts win{};

@@ -229,6 +229,76 @@ hg_status validate_ropes(const hg_grid_desc &D, const std::vector<int64_t> &leaf
 
 hg_status load_grid_impl(const hg_grid_desc *desc, const int32_t *ropes, int32_t validate_flag, hg_grid **out);
 
+// Whether every node bound is a single-precision number of the range that the single-precision records and
+// walks are made for (LeafRecF), and the links fit the nodes' fields.
+bool single_precision_bounds(const hg_grid_desc &D) {
+    if (D.n_nodes >= (1 << 29)) return false;
+    double most = 0.0;
+    for (int a = 0; a < 3; a++) most = std::max(most, std::max(std::fabs(D.node_lo[a]), std::fabs(D.node_hi[a])));
+    if (!(most >= 0x1p-20 && most <= 0x1p20)) return false;
+    auto fits = [](double v) {
+        const double m = std::fabs(v);
+        return v == 0.0 || (m >= 0x1p-60 && m <= 0x1p20 && (double)(float)v == v);
+    };
+    for (int64_t i = 0; i < 3 * D.n_nodes; i++)
+        if (!fits(D.node_lo[i]) || !fits(D.node_hi[i])) return false;
+    return true;
+}
+
+// Wall w of a leaf in its single-precision record: *first and the step bits (LeafRecF) from the wall's
+// neighbor list.
+uint32_t wall_slot(const hg_grid_desc &D, const std::vector<int64_t> &leaf_node, const std::vector<int32_t> &parent,
+                   int64_t leaf, int w, int32_t *first) {
+    const int64_t b0 = D.nbr_off[6 * leaf + w], cnt = D.nbr_off[6 * leaf + w + 1] - b0;
+    const int32_t *nb = D.nbr_id + b0;
+    *first = -1;
+    if (cnt <= 0) return 0;
+    *first = nb[0];
+    if (cnt == 1) return 0;
+    const int a = w >> 1, s = w & 1;
+    const int ax[2] = {a == 0 ? 1 : 0, a == 2 ? 1 : 2};
+    const double *flo = D.node_lo + 3 * leaf_node[(size_t)leaf], *fhi = D.node_hi + 3 * leaf_node[(size_t)leaf];
+    if (cnt == 2 || cnt == 4) {
+        int32_t at[4] = {-1, -1, -1, -1};  // leaf by its half on either axis
+        bool split[2] = {false, false}, ok = true;
+        for (int64_t j = 0; j < cnt && ok; j++) {
+            const double *lo = D.node_lo + 3 * leaf_node[(size_t)nb[j]], *hi = D.node_hi + 3 * leaf_node[(size_t)nb[j]];
+            int q = 0;
+            for (int b = 0; b < 2; b++) {
+                const double l = flo[ax[b]], h = fhi[ax[b]];
+                const double mid = 0.5f * ((float)l + (float)h);  // as the walk compares
+                if (lo[ax[b]] <= l && hi[ax[b]] >= h) continue;
+                split[b] = true;
+                if (lo[ax[b]] == mid && hi[ax[b]] >= h)
+                    q |= 1 << b;
+                else
+                    ok = ok && lo[ax[b]] <= l && hi[ax[b]] == mid;
+            }
+            ok = ok && at[q] < 0;
+            at[q] = nb[j];
+        }
+        ok = ok && at[0] >= 0 && (split[0] ? 2 : 1) * (split[1] ? 2 : 1) == cnt;
+        uint32_t bits = 0;
+        for (int b = 0; b < 2 && ok; b++) {
+            if (!split[b]) continue;
+            const int32_t step = at[1 << b] - at[0];
+            ok = at[1 << b] >= 0 && (step == 1 || step == 2 || step == 4);
+            bits |= (step == 1 ? 1u : step == 2 ? 2u : 3u) << (2 * b);
+        }
+        if (ok && cnt == 4) ok = at[3] == at[1] + at[2] - at[0];
+        if (ok) {
+            *first = at[0];
+            return bits << (4 * w);
+        }
+    }
+    // the rope node: the first ancestor of a neighbor that covers the face
+    const double P = s ? fhi[a] : flo[a];
+    int64_t nd = leaf_node[(size_t)nb[0]];
+    while (nd > 0 && !rope_covers(D, nd, a, s, P, flo, fhi)) nd = parent[(size_t)nd];
+    *first = (int32_t)(-2 - nd);
+    return 0;
+}
+
 }  // namespace
 
 extern "C" hg_status hg_build_ropes(const hg_grid_desc *desc, int32_t n_threads, int32_t *ropes) {
@@ -348,8 +418,37 @@ hg_status load_grid_impl(const hg_grid_desc *desc, const int32_t *ropes, int32_t
                     max_depth = std::max(max_depth, depth[i] + 1);
                 }
         // descent nodes
+        const bool f32 = single_precision_bounds(D);
         std::vector<unsigned char> nodes;
-        if (D.kind == HG_KDTREE) {
+        auto kd_axis = [&](int64_t i) {
+            const int64_t c = D.child_first[i];
+            int ax = 0;
+            while (ax < 2 && D.node_hi[3 * c + ax] == D.node_hi[3 * i + ax]) ax++;
+            return ax;
+        };
+        if (f32 && D.kind == HG_KDTREE) {
+            nodes.resize((size_t)(n + 1) * sizeof(hg::KdNodeF), 0);  // staged in whole 16-byte words
+            hg::KdNodeF *K = reinterpret_cast<hg::KdNodeF *>(nodes.data());
+            for (int64_t i = 0; i < n; i++) {
+                const int32_t c = D.child_first[i];
+                if (c < 0) {
+                    K[i].split = 0.0f;
+                    K[i].link = (uint32_t)D.node_leaf[i] << 2 | 3u;
+                } else {
+                    const int ax = kd_axis(i);
+                    K[i].split = (float)D.node_hi[3 * (int64_t)c + ax] + 0.0f;
+                    K[i].link = (uint32_t)c << 2 | (uint32_t)ax;
+                }
+            }
+        } else if (f32) {
+            nodes.resize((size_t)n * sizeof(hg::OctNodeF));
+            hg::OctNodeF *O = reinterpret_cast<hg::OctNodeF *>(nodes.data());
+            for (int64_t i = 0; i < n; i++) {
+                const int32_t c = D.child_first[i];
+                O[i].link = c < 0 ? -1 - D.node_leaf[i] : c;
+                for (int a = 0; a < 3; a++) O[i].s[a] = (c < 0) ? 0.0f : (float)D.node_hi[3 * (int64_t)c + a] + 0.0f;
+            }
+        } else if (D.kind == HG_KDTREE) {
             nodes.resize((size_t)n * sizeof(hg::KdNode));
             hg::KdNode *K = reinterpret_cast<hg::KdNode *>(nodes.data());
             for (int64_t i = 0; i < n; i++) {
@@ -359,8 +458,7 @@ hg_status load_grid_impl(const hg_grid_desc *desc, const int32_t *ropes, int32_t
                     K[i].split = 0;
                     K[i].info = D.node_leaf[i];
                 } else {
-                    int ax = 0;
-                    while (ax < 2 && D.node_hi[3 * (int64_t)c + ax] == D.node_hi[3 * i + ax]) ax++;
+                    const int ax = kd_axis(i);
                     K[i].split = hg::host_okey(D.node_hi[3 * (int64_t)c + ax]);
                     K[i].info = ax;
                 }
@@ -379,14 +477,15 @@ hg_status load_grid_impl(const hg_grid_desc *desc, const int32_t *ropes, int32_t
         std::vector<int64_t> leaf_node((size_t)nl);
         for (int64_t i = 0; i < n; i++)
             if (D.node_leaf[i] >= 0) leaf_node[D.node_leaf[i]] = i;
-        std::vector<hg::LeafRec> rec((size_t)nl);
+        std::vector<hg::LeafRec> rec(f32 ? 0 : (size_t)nl);
+        std::vector<hg::LeafRecF> recf(f32 ? (size_t)nl : 0);
         std::vector<int32_t> tail;
         int64_t long_walls = 0;
         // A list too long to scan keeps one tail entry instead: the wall's rope node (the deepest
         // node across the wall that covers the whole face), where the top-down search for the exit
         // point can start instead of the root.
         std::vector<int32_t> wall_ropes;
-        if (!ropes) {
+        if (!ropes && !f32) {
             bool any_long = false;
             for (int64_t i = 0; i < 6 * nl && !any_long; i++) any_long = D.nbr_off[i + 1] - D.nbr_off[i] > kScanLimit;
             if (any_long) {
@@ -396,7 +495,54 @@ hg_status load_grid_impl(const hg_grid_desc *desc, const int32_t *ropes, int32_t
             }
         }
         const double *dhi = D.node_hi;
-        for (int64_t i = 0; i < nl; i++) {
+        if (f32) {
+            std::vector<int32_t> parent;
+            if (!ropes) {
+                parent.assign((size_t)n, 0);
+                for (int64_t i = 0; i < n; i++)
+                    if (D.child_first[i] >= 0)
+                        for (int j = 0; j < nch; j++) parent[(size_t)D.child_first[i] + j] = (int32_t)i;
+            }
+            std::atomic<int64_t> next{0}, longs{0};
+            const int64_t chunk = 8192;
+            auto fill = [&]() {
+                for (;;) {
+                    const int64_t a0 = next.fetch_add(chunk);
+                    if (a0 >= nl) break;
+                    int64_t many = 0;
+                    for (int64_t i = a0; i < std::min(nl, a0 + chunk); i++) {
+                        hg::LeafRecF &R = recf[(size_t)i];
+                        const int64_t nd = leaf_node[(size_t)i];
+                        for (int a = 0; a < 3; a++) {  // + 0.0f: a bound of -0 is stored as +0
+                            R.lo[a] = (float)D.node_lo[3 * nd + a] + 0.0f;
+                            R.hi[a] = (float)D.node_hi[3 * nd + a] + 0.0f;
+                        }
+                        R.rho = D.leaf_rho[i];
+                        R.rho32 = (float)D.leaf_rho[i];
+                        R.steps = 0;
+                        for (int w = 0; w < 6; w++) {
+                            if (ropes) {
+                                R.first[w] = ropes[6 * i + w];
+                            } else {
+                                R.steps |= wall_slot(D, leaf_node, parent, i, w, &R.first[w]);
+                                many += D.nbr_off[6 * i + w + 1] - D.nbr_off[6 * i + w] > kScanLimit;
+                            }
+                        }
+                    }
+                    longs += many;
+                }
+            };
+            std::vector<std::thread> pool;
+            try {
+                const int threads = (int)std::min<int64_t>(std::max(1u, std::thread::hardware_concurrency()), nl / chunk);
+                for (int t = 1; t < threads; t++) pool.emplace_back(fill);
+            } catch (const std::system_error &) {  // fewer threads, then
+            }
+            fill();
+            for (auto &th : pool) th.join();
+            long_walls = longs;
+        }
+        for (int64_t i = 0; i < nl && !f32; i++) {
             hg::LeafRec &R = rec[i];
             std::memset(&R, 0, sizeof(R));
             const int64_t nd = leaf_node[i];
@@ -478,7 +624,9 @@ hg_status load_grid_impl(const hg_grid_desc *desc, const int32_t *ropes, int32_t
             if (r != cudaSuccess) return r;
             return cudaMemcpy(*dst, src, bytes, cudaMemcpyHostToDevice);
         };
-        if ((e = upload(&g->d_rec, rec.data(), rec.size() * sizeof(hg::LeafRec))) != cudaSuccess ||
+        const size_t rec_bytes = f32 ? recf.size() * sizeof(hg::LeafRecF) : rec.size() * sizeof(hg::LeafRec);
+        const void *rec_data = f32 ? static_cast<const void *>(recf.data()) : static_cast<const void *>(rec.data());
+        if ((e = upload(&g->d_rec, rec_data, rec_bytes)) != cudaSuccess ||
             (e = upload(&g->d_tail, tail.data(), tail.size() * sizeof(int32_t))) != cudaSuccess ||
             (e = upload(&g->d_nodes, nodes.data(), nodes.size())) != cudaSuccess ||
             (e = upload(&g->d_work, work.data(), work.size() * sizeof(float))) != cudaSuccess) {
@@ -487,7 +635,9 @@ hg_status load_grid_impl(const hg_grid_desc *desc, const int32_t *ropes, int32_t
             return st;
         }
         hg::DevGrid &G = g->d;
-        G.rec = static_cast<const hg::LeafRec *>(g->d_rec);
+        G.fdom = 0.0f;
+        G.rec = f32 ? nullptr : static_cast<const hg::LeafRec *>(g->d_rec);
+        G.recf = f32 ? static_cast<const hg::LeafRecF *>(g->d_rec) : nullptr;
         G.tail = static_cast<const int32_t *>(g->d_tail);
         G.nodes = g->d_nodes;
         G.work = static_cast<const float *>(g->d_work);
@@ -497,6 +647,9 @@ hg_status load_grid_impl(const hg_grid_desc *desc, const int32_t *ropes, int32_t
             G.dhi[a] = D.node_hi[a];
             G.klo[a] = hg::host_okey(G.dlo[a]);
             G.khi[a] = hg::host_okey(G.dhi[a]);
+            G.flo[a] = (float)G.dlo[a] + 0.0f;
+            G.fhi[a] = (float)G.dhi[a] + 0.0f;
+            G.fdom = std::max(G.fdom, std::max(std::fabs(G.flo[a]), std::fabs(G.fhi[a])));
         }
         G.n_leaves = nl;
         G.n_nodes = n;
@@ -504,14 +657,13 @@ hg_status load_grid_impl(const hg_grid_desc *desc, const int32_t *ropes, int32_t
         G.max_depth = max_depth;
         G.scan_limit = kScanLimit;
         G.nav = ropes ? HG_NAV_ROPES : HG_NAV_NEIGHBOR_LISTS;
-        G.pad = 0;
         hg_grid_info &I = g->info;
         I.kind = D.kind;
         I.max_depth = max_depth;
         I.n_nodes = n;
         I.n_leaves = nl;
         I.n_tail = (int64_t)tail.size();
-        I.device_bytes = (int64_t)(rec.size() * sizeof(hg::LeafRec) + tail.size() * 4 + nodes.size() +
+        I.device_bytes = (int64_t)(rec_bytes + tail.size() * 4 + nodes.size() +
                                    work.size() * sizeof(float));
         I.long_walls = long_walls;
         I.nav = ropes ? HG_NAV_ROPES : HG_NAV_NEIGHBOR_LISTS;

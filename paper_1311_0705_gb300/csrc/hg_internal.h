@@ -65,14 +65,51 @@ struct alignas(16) OctNode {
 };
 static_assert(sizeof(KdNode) == 16 && sizeof(OctNode) == 32, "node sizes");
 
+// The same for a grid whose node bounds are all single-precision numbers (zero, or of magnitude 2^-60 to
+// 2^20, the largest at least 2^-20): every dyadic tree of a domain such as [-1, 1]^3 down to level 23.  Bounds and split planes are
+// then held in single precision without loss, a leaf record is two 32-byte sectors instead of three --
+// one 64-byte DRAM access, where a 96-byte record always takes two -- and the walks decide most
+// crossings in single precision (walkf.cuh).  Grids with other bounds keep the records above.
+//   sector 0: lo.x lo.y lo.z hi.x hi.y hi.z (f32) rho
+//   sector 1: first[6] rho32 steps
+// first[w]: -1 when wall w lies on the domain boundary; the neighbor when one leaf covers the wall's face;
+// with steps bits 4w .. 4w+3 (e1 | e2 << 2) not zero, the leaf at the lower corner of the face, which two
+// or four equal leaves share, the leaf in the upper half on the first (second) of the two other axes
+// having an id higher by 2^(e1-1) (2^(e2-1)); otherwise -2 - the wall's rope node, the deepest node across
+// it that covers the face.  With HG_NAV_ROPES every wall of more than one neighbor holds its rope.
+struct alignas(32) LeafRecF {
+    float lo[3];
+    float hi[3];
+    double rho;
+    int32_t first[6];
+    float rho32;
+    uint32_t steps;
+};
+static_assert(sizeof(LeafRecF) == 64, "single-precision leaf record must be two sectors");
+
+// link = first child << 2 | split axis, or leaf << 2 | 3.
+struct alignas(8) KdNodeF {
+    float split;
+    uint32_t link;
+};
+// link = first child, or -1 - leaf.
+struct alignas(16) OctNodeF {
+    float s[3];
+    int32_t link;
+};
+static_assert(sizeof(KdNodeF) == 8 && sizeof(OctNodeF) == 16, "node sizes");
+
 // What a kernel needs to walk one grid (passed by value).
 struct DevGrid {
-    const LeafRec *rec;
+    const LeafRec *rec;     // or NULL: the records are recf, the nodes KdNodeF / OctNodeF
+    const LeafRecF *recf;
     const int32_t *tail;
     const void *nodes;
     const float *work;         // [work_n^3] expected crossings per unit length on a coarse lattice
     double dlo[3], dhi[3];
     long long klo[3], khi[3];  // keys of the domain bounds
+    float flo[3], fhi[3];      // the domain bounds (recf)
+    float fdom;                // the largest magnitude among them (recf)
     int64_t n_leaves;
     int64_t n_nodes;
     int32_t kind;
@@ -80,8 +117,11 @@ struct DevGrid {
     int32_t scan_limit;
     int32_t work_n;
     int32_t nav;  // HG_NAV_NEIGHBOR_LISTS or HG_NAV_ROPES: what the records' wall slots hold
-    int32_t pad;
 };
+inline int node_bytes_of(const DevGrid &G) {
+    if (G.recf) return G.kind == HG_KDTREE ? (int)sizeof(KdNodeF) : (int)sizeof(OctNodeF);
+    return G.kind == HG_KDTREE ? (int)sizeof(KdNode) : (int)sizeof(OctNode);
+}
 
 // Coarse lattice of the expected number of leaf crossings per unit path
 // length (volume average of S/(4V) over the leaves, Cauchy's mean chord),

@@ -4,7 +4,7 @@
 // runs inside a stream capture whose owner forbids allocation nodes,
 // real-time loops that must never enter an allocator, and hosts that give
 // this library a fixed memory budget up front.  hg_trace_rays takes its
-// scratch (a 48-byte start record per ray and a work counter) from the
+// scratch (a 48- or 64-byte start record per ray and a work counter) from the
 // stream-ordered allocator; this entry point takes it from one fixed array
 // compiled into the library instead, and allocates nothing.
 #include <cuda_runtime.h>
@@ -12,12 +12,12 @@
 #include <mutex>
 
 #include "hg_internal.h"
-#include "walk.cuh"
+#include "walkf.cuh"
 
 namespace hg {
 hg_status trace_rays_prealloc(const hg_grid *g, int64_t n, const double *o, const double *d, const double *s_max,
                               double kappa, const hg_trace_opts *opts, void *tau, int32_t *ncross,
-                              uint8_t *ray_status, RayStart *starts, unsigned long long *counter,
+                              uint8_t *ray_status, void *starts, unsigned long long *counter,
                               cudaStream_t stream);
 }
 
@@ -25,7 +25,8 @@ namespace {
 
 // Layout: the work counter in the first 256 bytes, then the start records.
 constexpr size_t kCounterBytes = 256;
-constexpr size_t kScratchBytes = kCounterBytes + (size_t)HG_NOALLOC_MAX_RAYS * sizeof(hg::RayStart);
+constexpr size_t kScratchBytes = kCounterBytes + (size_t)HG_NOALLOC_MAX_RAYS * sizeof(hg::RayStartF);
+static_assert(sizeof(hg::RayStartF) >= sizeof(hg::RayStart), "the scratch holds either start record");
 
 // Every GPU that loads the library holds this array until the process exits.
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
@@ -80,6 +81,6 @@ extern "C" hg_status hg_trace_rays_noalloc(const hg_grid *g, int64_t n, const do
     // the counter is zeroed by the launch itself (cudaMemsetAsync); the start
     // records are fully rewritten by the setup pass before they are read
     return hg::trace_rays_prealloc(g, n, o, d, s_max, kappa, opts, tau, ncross, ray_status,
-                                   reinterpret_cast<hg::RayStart *>(b + kCounterBytes),
+                                   b + kCounterBytes,
                                    reinterpret_cast<unsigned long long *>(b), (cudaStream_t)stream);
 }

@@ -1,75 +1,18 @@
 // Path-calculation kernels and their C entry points: optical depth and
 // crossing counts, segment emission, adjoint scatter, density sampling,
 // plus the small scan / reduction kernels the path needs.
-#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
 #include <mutex>
 #include <new>
+#include <type_traits>
 
 #include "hg_internal.h"
-#include "walk.cuh"
-
-namespace cg = cooperative_groups;
+#include "trace_args.cuh"
+#include "walkf.cuh"
 
 namespace hg {
-
-struct TraceArgs {
-    DevGrid G;
-    int64_t n;
-    const double *o;
-    const double *d;
-    const double *smax;
-    double kappa;
-    void *tau;
-    int32_t *ncross;
-    uint8_t *status;
-    const int64_t *seg_off;
-    int32_t *seg_cell;
-    void *seg_ds;
-    int64_t seg_cap;
-    const float *w;
-    void *grad;
-    uint32_t gmul, gmask;   // gradient slot of leaf c: (c * gmul) & gmask; gmul 0: slot c
-    const double *rho_ext;  // densities replacing the grid's own (MODE_TAU), or NULL
-    int64_t max_steps;
-    unsigned long long *counter;
-    const RayStart *starts;
-    const int64_t *order;  // queue position -> ray (most work first), or NULL
-    int n_smem;
-    int dyn;
-    // path segments of split rays (queue positions before the rays), or NULL
-    const unsigned long long *n_seg;
-    int64_t n_seg_cap;
-    const SegStart *segs;
-    double *part_acc;
-    int32_t *part_nc;
-    int32_t *part_last;
-    uint8_t *part_st;
-    const int64_t *seg_base;  // emission offset of each path segment (fill walks)
-    // emission staging (MODE_*_STAGE)
-    void *stg_ent;
-    uint32_t *stg_next;
-    uint32_t stg_nchunks;
-    unsigned long long *stg_ctr;
-    uint32_t *stg_start_ray;
-    uint32_t *stg_start_seg;
-    uint32_t *stg_overflow;
-    const uint32_t *run_if;  // when non-NULL, the walk runs only if *run_if != 0
-    // interaction points (MODE_INTERACT)
-    const double *tau_int;
-    int32_t *int_cell;
-    double *int_t;
-};
-
-// Stage the first n nodes of the (breadth-first) node list in shared memory.
-__device__ __forceinline__ void stage_nodes(const void *nodes, int bytes, unsigned char *smem) {
-    const int4 *src = reinterpret_cast<const int4 *>(nodes);
-    int4 *dst = reinterpret_cast<int4 *>(smem);
-    for (int i = threadIdx.x; i < bytes / 16; i += blockDim.x) dst[i] = __ldg(src + i);
-    __syncthreads();
-}
 
 // Setup pass: one ray per thread, every thread doing the same work (checks,
 // 1/d, clip, top-down location of the first leaf), so that the walking
@@ -83,6 +26,12 @@ __device__ __forceinline__ void stage_nodes(const void *nodes, int bytes, unsign
 // the dynamic queue hands out the heaviest paths first.
 constexpr int kBuckets = 32;
 
+template <int KIND, bool F>
+__host__ __device__ constexpr int node_size() {
+    return F ? (KIND == HG_KDTREE ? (int)sizeof(KdNodeF) : (int)sizeof(OctNodeF))
+             : (KIND == HG_KDTREE ? (int)sizeof(KdNode) : (int)sizeof(OctNode));
+}
+
 __device__ __forceinline__ int work_bucket(float w) {
     const int b = (int)(__log2f(1.0f + fmaxf(w, 0.0f)) * 3.0f);
     return kBuckets - 1 - (b < 0 ? 0 : (b > kBuckets - 1 ? kBuckets - 1 : b));  // 0 = most work
@@ -91,26 +40,39 @@ __device__ __forceinline__ int work_bucket(float w) {
 // With a non-NULL work_total the pass also adds up the rays' estimated work
 // (each rounded up to an integer, so the total does not depend on the order
 // of the additions); the split planner sizes path segments from it.
-template <int KIND>
+// F: the grid holds single-precision records; the start records are then RayStartF and t1, when not NULL,
+// receives the ends of the estimates' marches.
+template <int KIND, bool F>
 __global__ void __launch_bounds__(256) setup_kernel(const DevGrid G, int64_t n, const double *__restrict__ o,
                                                     const double *__restrict__ d, const double *__restrict__ smax,
-                                                    RayStart *starts, int n_smem, unsigned long long *bucket_count,
+                                                    void *starts, int n_smem, unsigned long long *bucket_count,
                                                     const int64_t *__restrict__ seg_off,
-                                                    unsigned long long *work_total, float *work) {
+                                                    unsigned long long *work_total, float *work, float *t1) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ unsigned int hist[kBuckets];
     if (threadIdx.x < kBuckets) hist[threadIdx.x] = 0;
-    const int node_bytes = n_smem * (KIND == HG_KDTREE ? 16 : 32);
+    const int node_bytes = n_smem * node_size<KIND, F>();
     // the work lattice follows the staged nodes when the pass estimates work
     const bool estimate = bucket_count != nullptr && !seg_off;
-    float *lat = (estimate && G.work) ? reinterpret_cast<float *>(smem + node_bytes) : nullptr;
+    float *lat = (estimate && G.work) ? reinterpret_cast<float *>(smem + geo_offset(node_bytes)) : nullptr;
     if (lat) stage_lattice(G, lat);
     stage_nodes(G.nodes, node_bytes, smem);
     unsigned long long wsum = 0;
     for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < n; r += (int64_t)gridDim.x * blockDim.x) {
-        RayStart R = ray_setup<KIND>(G, smem, n_smem, o, d, smax, r, estimate, lat);
+        RayStart R = ray_setup(
+            G,
+            [&](long long p0, long long p1, long long p2, uint32_t sg) {
+                return F ? locate_key_f<KIND>(G, smem, n_smem, p0, p1, p2, sg)
+                         : descend<KIND>(G, smem, n_smem, p0, p1, p2, sg);
+            },
+            o, d, smax, r, estimate, lat);
         if (seg_off) R.work = (float)(seg_off[r + 1] - seg_off[r]);
-        starts[r] = R;
+        if (F) {
+            static_cast<RayStartF *>(starts)[r] = start_f(R, o, d, r);
+            if (t1) t1[r] = R.t1;
+        } else {
+            static_cast<RayStart *>(starts)[r] = R;
+        }
         if (work) work[r] = R.work;
         if (bucket_count) atomicAdd(&hist[work_bucket(R.work)], 1u);
         wsum += (unsigned long long)ceilf(fmaxf(R.work, 0.0f));
@@ -175,14 +137,24 @@ struct SplitRec {
 // whole and the slots taken would be marked empty.
 constexpr int kPlanWarps = 8;  // warps per 256-thread block
 
-template <int KIND>
+__device__ __forceinline__ float start_work(const RayStart &R, const float *, int64_t) { return R.work; }
+__device__ __forceinline__ float start_work(const RayStartF &, const float *work, int64_t r) { return work[r]; }
+__device__ __forceinline__ float start_t1(const RayStart &R, const float *, int64_t) { return R.t1; }
+__device__ __forceinline__ float start_t1(const RayStartF &, const float *t1, int64_t r) { return t1[r]; }
+
+// F: single-precision records (the work estimates and march ends come from work and t1).
+template <int KIND, bool F>
 __global__ void __launch_bounds__(256) split_kernel(const DevGrid G, int64_t n, const double *__restrict__ o,
                                                     const double *__restrict__ d, const double *__restrict__ smax,
-                                                    RayStart *starts, int n_smem, const unsigned long long *work_total,
+                                                    void *starts_v, const float *__restrict__ work,
+                                                    const float *__restrict__ t1,
+                                                    const unsigned long long *work_total,
                                                     const unsigned long long *bucket_count,
                                                     const int64_t *__restrict__ order, int64_t threads, int force,
                                                     SegStart *segs, int64_t seg_cap, unsigned long long *seg_count,
                                                     SplitRec *list, unsigned long long *split_count) {
+    using Start = typename std::conditional<F, RayStartF, RayStart>::type;
+    Start *starts = static_cast<Start *>(starts_v);
     __shared__ int32_t s_leaf[kPlanWarps][kMaxSegs];
     __shared__ long long s_key[kPlanWarps][kMaxSegs];
     __shared__ long long s_ncand;
@@ -205,18 +177,19 @@ __global__ void __launch_bounds__(256) split_kernel(const DevGrid G, int64_t n, 
     const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
     float dom = 0.0f;
 #pragma unroll
-    for (int a = 0; a < 3; a++) dom = fmaxf(dom, fmaxf(fabsf((float)G.dlo[a]), fabsf((float)G.dhi[a])));
+    for (int a = 0; a < 3; a++) dom = fmaxf(dom, fmaxf(fabsf(G.flo[a]), fabsf(G.fhi[a])));
     for (int64_t q = (int64_t)blockIdx.x * (blockDim.x >> 5) + wib; q < ncand; q += nwarps) {
         const int64_t r = order[q];
-        const RayStart R = starts[r];
-        if (R.cur < 0 || !(R.work > thr)) continue;  // uniform over the warp
-        const int K = (int)fminf((float)kMaxSegs, ceilf(R.work / W));
+        const Start R = starts[r];
+        const float rwork = start_work(R, work, r);
+        if (R.cur < 0 || !(rwork > thr)) continue;  // uniform over the warp
+        const int K = (int)fminf((float)kMaxSegs, ceilf(rwork / W));
         const float of[3] = {(float)o[3 * r], (float)o[3 * r + 1], (float)o[3 * r + 2]};
         const float kf[3] = {(float)d[3 * r], (float)d[3 * r + 1], (float)d[3 * r + 2]};
         const uint32_t sg = R.sg & 0x3fu;
         // the walked interval as the setup's march took it: entry time to the domain exit or s_max
         const float ts = (float)kdouble(R.ktstart);
-        const float tend = R.t1;
+        const float tend = start_t1(R, t1, r);
         // cuts stay clear of both ends of the path
         const float lo_t = ts + (tend - ts) * 0x1p-10f, hi_t = tend - (tend - ts) * 0x1p-10f;
         // cut time of this lane: where the estimated work reaches (lane + 1) / K of the total.  The
@@ -233,8 +206,8 @@ __global__ void __launch_bounds__(256) split_kernel(const DevGrid G, int64_t n, 
             int ci[3];
 #pragma unroll
             for (int a = 0; a < 3; a++) {
-                const float lo = (float)G.dlo[a];
-                const float p = (of[a] + kf[a] * tm - lo) * ((float)N / ((float)G.dhi[a] - lo));
+                const float lo = G.flo[a];
+                const float p = (of[a] + kf[a] * tm - lo) * ((float)N / (G.fhi[a] - lo));
                 const int c = (int)floorf(p);
                 ci[a] = c < 0 ? 0 : (c > N - 1 ? N - 1 : c);
             }
@@ -262,25 +235,34 @@ __global__ void __launch_bounds__(256) split_kernel(const DevGrid G, int64_t n, 
         bool ok = false;
         int32_t Lid = -1;
         if (lane < K - 1 && found && tc > lo_t && tc < hi_t) {
-            long long q3[3], qm[3], qp[3];
+            long long q3[3];
+            float xm[3], xp[3];
 #pragma unroll
             for (int a = 0; a < 3; a++) {
                 const float x = of[a] + kf[a] * tc;
                 const float m = (fabsf(of[a]) + fabsf(kf[a] * tc) + dom) * 0x1p-18f;
                 q3[a] = f32_key(x);
-                qm[a] = f32_key(x - m);
-                qp[a] = f32_key(x + m);
+                xm[a] = x - m;
+                xp[a] = x + m;
             }
             if (in_axis(q3[0], G.klo[0], G.khi[0], dpos(sg, 0), dneg(sg, 0), true) &&
                 in_axis(q3[1], G.klo[1], G.khi[1], dpos(sg, 1), dneg(sg, 1), true) &&
                 in_axis(q3[2], G.klo[2], G.khi[2], dpos(sg, 2), dneg(sg, 2), true))
-                Lid = descend<KIND>(G, nullptr, 0, q3[0], q3[1], q3[2], sg);
+                Lid = F ? locate_key_f<KIND>(G, nullptr, 0, q3[0], q3[1], q3[2], sg)
+                        : descend<KIND>(G, nullptr, 0, q3[0], q3[1], q3[2], sg);
             if (Lid >= 0) {
-                Leaf L;
-                load_leaf(G.rec, Lid, L);
                 ok = true;
+                if (F) {
+                    const LeafRecF *L = G.recf + Lid;
 #pragma unroll
-                for (int a = 0; a < 3; a++) ok = ok && qm[a] >= L.lo(a) && qp[a] <= L.hi(a);
+                    for (int a = 0; a < 3; a++) ok = ok && xm[a] >= __ldg(&L->lo[a]) && xp[a] <= __ldg(&L->hi[a]);
+                } else {
+                    Leaf L;
+                    load_leaf(G.rec, Lid, L);
+#pragma unroll
+                    for (int a = 0; a < 3; a++)
+                        ok = ok && f32_key(xm[a]) >= L.lo(a) && f32_key(xp[a]) <= L.hi(a);
+                }
             }
         }
         // accept cuts in path order: increasing t_c, a leaf different from the previous cut's
@@ -316,6 +298,10 @@ __global__ void __launch_bounds__(256) split_kernel(const DevGrid G, int64_t n, 
                 E.cur = -1;
                 E.sg = 0;
                 segs[s] = E;
+                if constexpr (F) {
+                    starts[n + (int64_t)s].cur = -1;
+                    starts[n + (int64_t)s].sg = 0;
+                }
             }
             continue;
         }
@@ -327,6 +313,13 @@ __global__ void __launch_bounds__(256) split_kernel(const DevGrid G, int64_t n, 
             E.cur = lane == 0 ? R.cur : s_leaf[wib][lane - 1];
             E.sg = sg | (lane == 0 ? 0u : SG_SKIP_FIRST);
             segs[first + lane] = E;
+            if constexpr (F) {  // the segment's start record
+                RayStartF B = R;
+                B.ktstart = E.ktstart;
+                B.cur = E.cur;
+                B.sg = E.sg | (R.sg & SG_EXACT);
+                starts[n + (int64_t)first + lane] = B;
+            }
         }
         if (lane == 0) {
             const unsigned long long i = atomicAdd(split_count, 1ULL);
@@ -435,49 +428,6 @@ __global__ void __launch_bounds__(256) order_kernel(int64_t n, const float *__re
     }
 }
 
-// Rays of one grid for the walking loop: a static stride, or a
-// warp-aggregated atomic on a global counter.
-struct GridRays {
-    static constexpr bool kSegments = true;
-    const DevGrid *G;
-    int64_t n;
-    int64_t cursor;
-    int64_t stride;
-    unsigned long long *counter;
-    const int64_t *order;
-    int64_t n_seg;  // queue positions 0 .. n_seg-1 are path segments (items n + s)
-    int32_t max_steps;
-    bool dyn;
-    __device__ __forceinline__ bool next(int64_t &ray, const DevGrid *&g, int32_t &ms) {
-        g = G;
-        ms = max_steps;
-        if (dyn) {
-            cg::coalesced_group grp = cg::coalesced_threads();
-            unsigned long long base = 0;
-            if (grp.thread_rank() == 0) base = atomicAdd(counter, (unsigned long long)grp.size());
-            base = grp.shfl(base, 0);
-            int64_t pos = (int64_t)(base + grp.thread_rank());
-            if (pos < n_seg) {
-                ray = n + pos;
-                return true;
-            }
-            pos -= n_seg;
-            ray = (pos < n && order) ? order[pos] : pos;
-            return pos < n;
-        }
-        ray = cursor;
-        cursor += stride;
-        return ray < n;
-    }
-};
-
-// Dynamic shared memory of a walking launch: the top tree nodes, then the
-// threads' geometry slots (9 doubles per thread) at a 16-byte boundary.
-__host__ __device__ __forceinline__ size_t geo_offset(size_t node_bytes) { return (node_bytes + 15) / 16 * 16; }
-__host__ __device__ __forceinline__ size_t walk_smem(size_t node_bytes, int block) {
-    return geo_offset(node_bytes) + (size_t)block * 9 * sizeof(double);
-}
-
 // One persistent loop per thread (walk_loop): a lane whose ray has ended
 // takes the next one, and every iteration advances each lane by one record
 // load, so lanes never wait for the longest path in their warp.
@@ -490,64 +440,14 @@ __global__ void __launch_bounds__(256, OCC) trace_kernel(const TraceArgs A) {
     if (A.run_if && *A.run_if == 0u) return;  // a fallback walk with nothing to do
     const int node_bytes = (KIND == HG_KDTREE) ? 16 : 32;
     stage_nodes(A.G.nodes, A.n_smem * node_bytes, smem);
-    GridRays src;
-    src.G = &A.G;
-    src.n = A.n;
-    src.cursor = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    src.stride = (int64_t)gridDim.x * blockDim.x;
-    src.counter = A.counter;
-    src.order = A.order;
-    src.max_steps = (int32_t)(A.max_steps < 0x7fffffff ? A.max_steps : 0x7fffffff);
-    src.dyn = A.dyn != 0;
-    src.n_seg = 0;
-    if (A.n_seg && src.dyn) {
-        const unsigned long long c = *A.n_seg;
-        src.n_seg = (int64_t)(c < (unsigned long long)A.n_seg_cap ? c : (unsigned long long)A.n_seg_cap);
-    }
+    GridRays src(A);
     WalkIO io;
-    io.o = A.o;
-    io.d = A.d;
-    io.smax = A.smax;
-    io.starts = A.starts;
-    io.kappa = A.kappa;
-    io.tau = A.tau;
-    io.ncross = A.ncross;
-    io.status = A.status;
-    io.seg_off = A.seg_off;
-    io.seg_cell = A.seg_cell;
-    io.seg_ds = A.seg_ds;
-    io.seg_cap = A.seg_cap;
-    io.w = A.w;
-    io.grad = A.grad;
-    if (A.gmul) {
-        io.gmul = A.gmul;
-        io.gmask = A.gmask;
-    }
-    io.rho_ext = A.rho_ext;
-    io.n_rays = A.n;
-    io.segs = A.segs;
-    io.part_acc = A.part_acc;
-    io.part_nc = A.part_nc;
-    io.part_last = A.part_last;
-    io.part_st = A.part_st;
-    io.seg_base = A.seg_base;
-    io.stg_ent = A.stg_ent;
-    io.stg_next = A.stg_next;
-    io.stg_nchunks = A.stg_nchunks;
-    io.stg_ctr = A.stg_ctr;
-    io.stg_start_ray = A.stg_start_ray;
-    io.stg_start_seg = A.stg_start_seg;
-    io.stg_overflow = A.stg_overflow;
-    io.tau_int = A.tau_int;
-    io.int_cell = A.int_cell;
-    io.int_t = A.int_t;
+    walk_io(A, io);
     walk_loop<KIND, MODE, PREC, NAV>(src, io, smem, A.n_smem,
                                      reinterpret_cast<double *>(smem + geo_offset(A.n_smem * node_bytes)));
 }
 
 // ------------------------------------------------------------------ launch plumbing
-
-typedef void (*KernelFn)(const TraceArgs);
 
 // Walking kernels by [navigation][kind][mode][prec][occupancy]; prec runs
 // 0..1, and 0..3 for MODE_TAUADJ and MODE_TAUADJ_STAGE (optical depth and
@@ -600,7 +500,7 @@ int sm_count() {
 // rays took 0.52 ms against 0.29 ms.
 constexpr int kWalkNodes = 64;
 int setup_nodes(const hg_grid *g) {
-    const int node_bytes = g->d.kind == HG_KDTREE ? 16 : 32;
+    const int node_bytes = node_bytes_of(g->d);
     return (int)std::min<int64_t>(g->d.n_nodes, (8 * 1024) / node_bytes);
 }
 
@@ -637,14 +537,21 @@ hg_status resolve_opts(const hg_grid *g, const hg_trace_opts *opts, int &precisi
         return HG_EINVAL;
     }
     // clamp to the node count and to 200 KB of shared memory
-    const int node_bytes = g->d.kind == HG_KDTREE ? 16 : 32;
+    const int node_bytes = node_bytes_of(g->d);
     smem_nodes = (int)std::min<int64_t>(std::min<int64_t>(smem_nodes, g->d.n_nodes), (200 * 1024) / node_bytes);
     return HG_OK;
 }
 
 constexpr int kLatticeBytes = kWorkN * kWorkN * kWorkN * (int)sizeof(float);
-constexpr int kWalkSmemMax = 200 * 1024 + 256 * 9 * (int)sizeof(double);
+constexpr int kWalkSmemMax = 200 * 1024 + 256 * kGeoBytes;
 constexpr int kSetupSmemMax = 200 * 1024 + kLatticeBytes;
+
+using SetupFn = void (*)(const DevGrid, int64_t, const double *, const double *, const double *, void *, int,
+                         unsigned long long *, const int64_t *, unsigned long long *, float *, float *);
+SetupFn pick_setup(int kind, bool f) {
+    if (f) return kind == HG_KDTREE ? &setup_kernel<HG_KDTREE, true> : &setup_kernel<HG_OCTREE, true>;
+    return kind == HG_KDTREE ? &setup_kernel<HG_KDTREE, false> : &setup_kernel<HG_OCTREE, false>;
+}
 
 void set_smem_limits() {
     static std::once_flag once;
@@ -657,12 +564,25 @@ void set_smem_limits() {
                             cudaFuncSetAttribute(pick_kernel(kd, m, p, oc, nav),
                                                  cudaFuncAttributeMaxDynamicSharedMemorySize, kWalkSmemMax);
         // the setup pass also stages the work lattice after the nodes
-        cudaFuncSetAttribute(setup_kernel<HG_KDTREE>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSetupSmemMax);
-        cudaFuncSetAttribute(setup_kernel<HG_OCTREE>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSetupSmemMax);
+        for (int kd = 0; kd < 2; kd++)
+            for (int f = 0; f < 2; f++)
+                cudaFuncSetAttribute(pick_setup(kd, f != 0), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     kSetupSmemMax);
     });
 }
 
-// Resident blocks of a walking kernel for a launch shape.
+// The walking kernel for a grid.  Grids with single-precision records have one variant per mode (either
+// tree and navigation, 64 registers): their tree descents are rare and read the node format at run time.
+KernelFn walk_kernel(const hg_grid *g, int mode, int prec, int occ) {
+    return g->d.recf ? pick_kernel_f(mode, prec) : pick_kernel(g->d.kind, mode, prec, occ, g->d.nav);
+}
+size_t walk_smem_of(const hg_grid *g, int smem_nodes, int block) {
+    return g->d.recf ? walk_smem_f(block) : walk_smem((size_t)smem_nodes * node_bytes_of(g->d), block);
+}
+
+// Blocks of a walking launch of n items on grid g, at most those resident.  On single-precision grids a
+// warp shares its items out among its lanes: down to one item per warp the launch takes another block.
+int64_t walk_items(const hg_grid *g, int64_t n) { return g->d.recf && n < INT64_MAX / 64 ? n * 32 : n; }
 hg_status walk_blocks(KernelFn k, int block, size_t smem, int64_t n, int64_t &blocks) {
     int per_sm = 0;
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, block, smem);
@@ -688,12 +608,11 @@ struct hg_rays {
     int64_t max_steps = 0, threads = 0;
     bool dyn = false, ordered = false, splitting = false;
     bool traced = false;  // an optical-depth walk recorded the segments' crossing counts
-    size_t smem = 0;       // top tree nodes (the setup pass)
     size_t walk_smem = 0;  // top tree nodes and the threads' ray geometry (the walks)
     unsigned char *scratch = nullptr;
-    hg::RayStart *starts = nullptr;
+    void *starts = nullptr;  // RayStart, or RayStartF on a grid with single-precision records
     int64_t *order = nullptr;
-    float *work = nullptr;
+    float *work = nullptr, *t1 = nullptr;
     unsigned long long *counts = nullptr, *work_total = nullptr, *seg_count = nullptr, *split_count = nullptr,
                        *queue = nullptr;
     hg::SegStart *segs = nullptr;
@@ -735,11 +654,10 @@ hg_status make_plan(hg_rays &P, const hg_grid *g, int64_t n, const double *o, co
     P.smem_nodes = smem_nodes;
     P.min_blocks = min_blocks;
     P.max_steps = max_steps;
-    const int node_bytes = g->d.kind == HG_KDTREE ? 16 : 32;
-    P.smem = (size_t)smem_nodes * node_bytes;
-    P.walk_smem = walk_smem(P.smem, block);
+    const bool f32 = g->d.recf != nullptr;
+    P.walk_smem = walk_smem_of(g, smem_nodes, block);
     int64_t blocks = 0;
-    const KernelFn k0 = pick_kernel(g->d.kind, MODE_TAU, HG_FP64, min_blocks, g->d.nav);
+    const KernelFn k0 = walk_kernel(g, MODE_TAU, HG_FP64, min_blocks);
     hg_status hs = walk_blocks(k0, block, P.walk_smem, n, blocks);
     if (hs != HG_OK) return hs;
     P.threads = blocks * block;
@@ -761,7 +679,9 @@ hg_status make_plan(hg_rays &P, const hg_grid *g, int64_t n, const double *o, co
     // total, segment and split-ray counts); for splitting the segment
     // records, partial results, emission offsets and the list of split rays
     auto al = [](size_t b) { return (b + 255) / 256 * 256; };
-    const size_t start_bytes = al((size_t)n * sizeof(RayStart));
+    // (single-precision grids: start records of the segments after those of the rays)
+    const size_t start_bytes = al(f32 ? (size_t)(n + P.seg_cap) * sizeof(RayStartF) : (size_t)n * sizeof(RayStart));
+    const size_t t1_bytes = P.splitting && f32 ? al((size_t)n * sizeof(float)) : 0;
     const size_t order_bytes = P.ordered ? al((size_t)n * sizeof(int64_t)) : 0;
     const size_t work_bytes = P.ordered ? al((size_t)n * sizeof(float)) : 0;
     const size_t count_bytes = al((2 * kBuckets + 4) * sizeof(unsigned long long));
@@ -772,7 +692,7 @@ hg_status make_plan(hg_rays &P, const hg_grid *g, int64_t n, const double *o, co
     const size_t base_bytes = al((size_t)P.seg_cap * sizeof(int64_t));
     const size_t list_bytes = al((size_t)(P.seg_cap / 2) * sizeof(SplitRec));
     const size_t total_bytes = start_bytes + order_bytes + work_bytes + count_bytes + seg_bytes + acc_bytes +
-                               2 * i32_bytes + u8_bytes + base_bytes + list_bytes;
+                               2 * i32_bytes + u8_bytes + base_bytes + list_bytes + t1_bytes;
     cudaError_t e = cudaMallocAsync((void **)&P.scratch, total_bytes, stream);
     if (e != cudaSuccess) {
         P.scratch = nullptr;
@@ -784,7 +704,7 @@ hg_status make_plan(hg_rays &P, const hg_grid *g, int64_t n, const double *o, co
         off += b;
         return q;
     };
-    P.starts = reinterpret_cast<RayStart *>(take(start_bytes));
+    P.starts = take(start_bytes);
     P.order = reinterpret_cast<int64_t *>(take(order_bytes));
     P.work = reinterpret_cast<float *>(take(work_bytes));
     unsigned long long *cnt = reinterpret_cast<unsigned long long *>(take(count_bytes));
@@ -795,6 +715,7 @@ hg_status make_plan(hg_rays &P, const hg_grid *g, int64_t n, const double *o, co
     P.part_st = reinterpret_cast<uint8_t *>(take(u8_bytes));
     P.seg_base = reinterpret_cast<int64_t *>(take(base_bytes));
     P.list = reinterpret_cast<SplitRec *>(take(list_bytes));
+    P.t1 = reinterpret_cast<float *>(take(t1_bytes));
     P.counts = P.ordered ? cnt : nullptr;
     P.work_total = cnt + 2 * kBuckets;
     P.seg_count = cnt + 2 * kBuckets + 1;
@@ -804,13 +725,10 @@ hg_status make_plan(hg_rays &P, const hg_grid *g, int64_t n, const double *o, co
     if (e != cudaSuccess) return cuda_err(e, "scratch reset");
     const int64_t sblocks = std::min<int64_t>((n + 255) / 256, (int64_t)sm_count() * 8);
     const int snodes = setup_nodes(g);
-    const size_t setup_smem = (size_t)snodes * node_bytes + ((P.ordered && !exact && g->d.work) ? kLatticeBytes : 0);
-    if (g->d.kind == HG_KDTREE)
-        setup_kernel<HG_KDTREE><<<(unsigned)sblocks, 256, setup_smem, stream>>>(
-            g->d, n, o, d, smax, P.starts, snodes, P.counts, exact, P.ordered ? P.work_total : nullptr, P.work);
-    else
-        setup_kernel<HG_OCTREE><<<(unsigned)sblocks, 256, setup_smem, stream>>>(
-            g->d, n, o, d, smax, P.starts, snodes, P.counts, exact, P.ordered ? P.work_total : nullptr, P.work);
+    const size_t setup_smem = geo_offset((size_t)snodes * node_bytes_of(g->d)) +
+                              ((P.ordered && !exact && g->d.work) ? kLatticeBytes : 0);
+    pick_setup(g->d.kind, f32)<<<(unsigned)sblocks, 256, setup_smem, stream>>>(
+        g->d, n, o, d, smax, P.starts, snodes, P.counts, exact, P.ordered ? P.work_total : nullptr, P.work, P.t1);
     note_launches(1);
     if (P.ordered) {
         order_kernel<<<(unsigned)sblocks, 256, 0, stream>>>(n, P.work, P.counts, P.counts + kBuckets, P.order);
@@ -820,14 +738,13 @@ hg_status make_plan(hg_rays &P, const hg_grid *g, int64_t n, const double *o, co
         const int force = split == HG_SPLIT_FORCE ? 1 : 0;
         // one warp per candidate ray: as many blocks as are resident at once
         const unsigned pblocks = (unsigned)sm_count() * 4;
-        if (g->d.kind == HG_KDTREE)
-            split_kernel<HG_KDTREE><<<pblocks, 256, 0, stream>>>(
-                g->d, n, o, d, smax, P.starts, smem_nodes, P.work_total, P.counts, P.order, P.threads, force, P.segs,
-                P.seg_cap, P.seg_count, P.list, P.split_count);
-        else
-            split_kernel<HG_OCTREE><<<pblocks, 256, 0, stream>>>(
-                g->d, n, o, d, smax, P.starts, smem_nodes, P.work_total, P.counts, P.order, P.threads, force, P.segs,
-                P.seg_cap, P.seg_count, P.list, P.split_count);
+        const auto split_fn = f32 ? (g->d.kind == HG_KDTREE ? &split_kernel<HG_KDTREE, true>
+                                                            : &split_kernel<HG_OCTREE, true>)
+                                  : (g->d.kind == HG_KDTREE ? &split_kernel<HG_KDTREE, false>
+                                                            : &split_kernel<HG_OCTREE, false>);
+        split_fn<<<pblocks, 256, 0, stream>>>(g->d, n, o, d, smax, P.starts, P.work, P.t1, P.work_total, P.counts,
+                                              P.order, P.threads, force, P.segs, P.seg_cap, P.seg_count, P.list,
+                                              P.split_count);
         note_launches(1);
     }
     e = cudaGetLastError();
@@ -991,7 +908,7 @@ __device__ __forceinline__ bool copy_staged_group(uint32_t e, int64_t cnt, int64
 // Does nothing when the pool overflowed (the walks that follow then do the
 // emission and the adjoint).
 template <int GP, typename DS>
-__global__ void __launch_bounds__(256) gather_kernel(int64_t n, const RayStart *__restrict__ starts,
+__global__ void __launch_bounds__(256) gather_kernel(int64_t n, const uint32_t *__restrict__ start_sg, int sg_stride,
                                                      const int64_t *__restrict__ seg_off,
                                                      const uint32_t *__restrict__ start_ray,
                                                      const SplitRec *__restrict__ list,
@@ -1017,7 +934,7 @@ __global__ void __launch_bounds__(256) gather_kernel(int64_t n, const RayStart *
         int64_t cnt = 0, b = 0;
         uint32_t first = 0;
         double wk = 0.0;
-        if (r < n && !(starts[r].sg & SG_SPLIT)) {
+        if (r < n && !(start_sg[r * sg_stride] & SG_SPLIT)) {
             b = seg_off[r];
             cnt = seg_off[r + 1] - b;
             if (cnt > 0) {
@@ -1102,9 +1019,9 @@ __global__ void __launch_bounds__(256) gather_kernel(int64_t n, const RayStart *
 hg_status walk_plan(hg_rays &P, int mode, int prec, TraceArgs A, cudaStream_t stream) {
     if (P.n == 0) return HG_OK;
     const hg_grid *g = P.g;
-    KernelFn k = pick_kernel(g->d.kind, mode, prec, P.min_blocks, g->d.nav);
+    KernelFn k = walk_kernel(g, mode, prec, P.min_blocks);
     int64_t blocks = 0;
-    hg_status hs = walk_blocks(k, P.block, P.walk_smem, P.splitting ? INT64_MAX / 2 : P.n, blocks);
+    hg_status hs = walk_blocks(k, P.block, P.walk_smem, P.splitting ? INT64_MAX / 2 : walk_items(g, P.n), blocks);
     if (hs != HG_OK) return hs;
     A.G = g->d;
     A.n = P.n;
@@ -1210,20 +1127,20 @@ hg_status check_rays(const hg_grid *g, int64_t n, const double *o, const double 
 
 // ------------------------------------------------------------------ density sampling
 
-template <int KIND>
+template <int KIND, bool F>
 __global__ void sample_kernel(const DevGrid G, int64_t n, const double *__restrict__ pts, int32_t *cell,
                               double *rho, int n_smem) {
     extern __shared__ __align__(16) unsigned char smem[];
-    stage_nodes(G.nodes, n_smem * (KIND == HG_KDTREE ? 16 : 32), smem);
+    stage_nodes(G.nodes, n_smem * node_size<KIND, F>(), smem);
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const long long p0 = okey(pts[3 * i]), p1 = okey(pts[3 * i + 1]), p2 = okey(pts[3 * i + 2]);
         int32_t c = -1;
         // a point query uses the half-open rule of a zero direction
         if (in_axis(p0, G.klo[0], G.khi[0], false, false, true) && in_axis(p1, G.klo[1], G.khi[1], false, false, true) &&
             in_axis(p2, G.klo[2], G.khi[2], false, false, true))
-            c = descend<KIND>(G, smem, n_smem, p0, p1, p2, 0u);
+            c = F ? locate_key_f<KIND>(G, smem, n_smem, p0, p1, p2, 0u) : descend<KIND>(G, smem, n_smem, p0, p1, p2, 0u);
         if (cell) cell[i] = c;
-        rho[i] = (c >= 0) ? __ldg(&G.rec[c].rho) : 0.0;
+        rho[i] = (c >= 0) ? __ldg(F ? &G.recf[c].rho : &G.rec[c].rho) : 0.0;
     }
 }
 
@@ -1644,9 +1561,13 @@ static hg_status emit_staged(const char *name, hg_rays *r, const int64_t *seg_of
     }
     const int64_t gblocks = std::min<int64_t>((r->n * 8 + 255) / 256, (int64_t)sm_count() * 8);
     const unsigned long long *sc = r->splitting ? r->split_count : nullptr;
+    const bool f32 = r->g->d.recf != nullptr;
+    const uint32_t *start_sg = f32 ? &static_cast<const RayStartF *>(r->starts)->sg
+                                   : &static_cast<const RayStart *>(r->starts)->sg;
+    const int sg_stride = (int)((f32 ? sizeof(RayStartF) : sizeof(RayStart)) / sizeof(uint32_t));
 #define HG_GATHER(GP, DS)                                                                                          \
     gather_kernel<GP, DS><<<(unsigned)gblocks, 256, 0, s>>>(                                                     \
-        r->n, r->starts, seg_off, r->stg_start_ray, r->list, sc, r->stg_start_seg, r->part_nc, r->stg_ent,      \
+        r->n, start_sg, sg_stride, seg_off, r->stg_start_ray, r->list, sc, r->stg_start_seg, r->part_nc, r->stg_ent,      \
         r->stg_next, r->stg_overflow, seg_cell, static_cast<DS *>(seg_ds), seg_capacity, ray_status, kappa, w,  \
         B.grad, B.gmul, B.gmask)
     if (r->stg_prec == HG_FP64) {
@@ -1765,17 +1686,14 @@ extern "C" hg_status hg_sample_density(const hg_grid *g, int64_t n, const double
         return HG_EINVAL;
     }
     if (n == 0) return HG_OK;
-    const int node_bytes = g->d.kind == HG_KDTREE ? 16 : 32;
-    const int n_smem = (int)std::min<int64_t>(g->d.n_nodes, (8 * 1024) / node_bytes);
-    const size_t smem = (size_t)n_smem * node_bytes;
+    const int n_smem = setup_nodes(g);
+    const size_t smem = geo_offset((size_t)n_smem * node_bytes_of(g->d));
     const int block = 256;
     int64_t blocks = std::min<int64_t>((n + block - 1) / block, (int64_t)sm_count() * 8);
-    if (g->d.kind == HG_KDTREE)
-        sample_kernel<HG_KDTREE><<<(unsigned)blocks, block, smem, (cudaStream_t)stream>>>(g->d, n, pts, cell, rho,
-                                                                                         n_smem);
-    else
-        sample_kernel<HG_OCTREE><<<(unsigned)blocks, block, smem, (cudaStream_t)stream>>>(g->d, n, pts, cell, rho,
-                                                                                         n_smem);
+    const auto fn = g->d.recf ? (g->d.kind == HG_KDTREE ? &sample_kernel<HG_KDTREE, true> : &sample_kernel<HG_OCTREE, true>)
+                              : (g->d.kind == HG_KDTREE ? &sample_kernel<HG_KDTREE, false>
+                                                        : &sample_kernel<HG_OCTREE, false>);
+    fn<<<(unsigned)blocks, block, smem, (cudaStream_t)stream>>>(g->d, n, pts, cell, rho, n_smem);
     note_launches(1);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? HG_OK : cuda_err(e, "sample launch");
@@ -1844,7 +1762,7 @@ namespace hg {
 // stream-ordered allocator.  Used by the allocation-free entry point.
 hg_status trace_rays_prealloc(const hg_grid *g, int64_t n, const double *o, const double *d, const double *s_max,
                               double kappa, const hg_trace_opts *opts, void *tau, int32_t *ncross,
-                              uint8_t *ray_status, RayStart *starts, unsigned long long *counter,
+                              uint8_t *ray_status, void *starts, unsigned long long *counter,
                               cudaStream_t stream) {
     hg_status st = check_rays(g, n, o, d);
     if (st != HG_OK) return st;
@@ -1871,17 +1789,12 @@ hg_status trace_rays_prealloc(const hg_grid *g, int64_t n, const double *o, cons
     A.dyn = (schedule == 2);
     A.starts = starts;
     A.counter = counter;
-    KernelFn k = pick_kernel(g->d.kind, MODE_TAU, prec, min_blocks, g->d.nav);
-    const int node_bytes = g->d.kind == HG_KDTREE ? 16 : 32;
-    const size_t smem = (size_t)smem_nodes * node_bytes;
-    const size_t wsmem = walk_smem(smem, block);
+    const bool f32 = g->d.recf != nullptr;
+    KernelFn k = walk_kernel(g, MODE_TAU, prec, min_blocks);
+    const size_t wsmem = walk_smem_of(g, smem_nodes, block);
     cudaError_t e = cudaSuccess;
     if (wsmem > 48 * 1024) {
         e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kWalkSmemMax);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(setup_kernel<HG_KDTREE>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(setup_kernel<HG_OCTREE>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
         if (e != cudaSuccess) return cuda_err(e, "shared-memory limit of the allocation-free walk");
     }
     int per_sm = 0;
@@ -1891,20 +1804,16 @@ hg_status trace_rays_prealloc(const hg_grid *g, int64_t n, const double *o, cons
         set_error("launch shape does not fit on an SM (block %d, %zu B shared)", block, wsmem);
         return HG_EINVAL;
     }
-    int64_t blocks = std::min<int64_t>((int64_t)per_sm * sm_count(), (n + block - 1) / block);
+    int64_t blocks = std::min<int64_t>((int64_t)per_sm * sm_count(), (walk_items(g, n) + block - 1) / block);
     if (A.dyn) {
         e = cudaMemsetAsync(counter, 0, sizeof(unsigned long long), stream);
         if (e != cudaSuccess) return cuda_err(e, "counter reset");
     }
     const int64_t sblocks = std::min<int64_t>((n + 255) / 256, (int64_t)sm_count() * 8);
     const int snodes = setup_nodes(g);
-    const size_t ssmem = (size_t)snodes * node_bytes;
-    if (g->d.kind == HG_KDTREE)
-        setup_kernel<HG_KDTREE><<<(unsigned)sblocks, 256, ssmem, stream>>>(g->d, n, o, d, s_max, starts, snodes,
-                                                                          nullptr, nullptr, nullptr, nullptr);
-    else
-        setup_kernel<HG_OCTREE><<<(unsigned)sblocks, 256, ssmem, stream>>>(g->d, n, o, d, s_max, starts, snodes,
-                                                                          nullptr, nullptr, nullptr, nullptr);
+    const size_t ssmem = geo_offset((size_t)snodes * node_bytes_of(g->d));
+    pick_setup(g->d.kind, f32)<<<(unsigned)sblocks, 256, ssmem, stream>>>(g->d, n, o, d, s_max, starts, snodes, nullptr,
+                                                                         nullptr, nullptr, nullptr, nullptr);
     k<<<(unsigned)blocks, block, wsmem, stream>>>(A);
     note_launches(2);
     e = cudaGetLastError();

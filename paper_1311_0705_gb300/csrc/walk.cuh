@@ -258,8 +258,8 @@ __device__ __forceinline__ float work_march(const DevGrid &G, const float *lat, 
     int c[3], step[3];
 #pragma unroll
     for (int a = 0; a < 3; a++) {
-        const float lo = (float)G.dlo[a];
-        const float sc = (float)N / ((float)G.dhi[a] - lo);
+        const float lo = G.flo[a];
+        const float sc = (float)N / (G.fhi[a] - lo);
         const float ka = k[a] * sc;  // lattice units per unit t
         const float p = (o[a] + k[a] * t0 - lo) * sc;
         int ci = (int)floorf(p);
@@ -297,6 +297,17 @@ __device__ __forceinline__ float work_march(const DevGrid &G, const float *lat, 
     return e;
 }
 
+// Nearest single-precision value of a double (half away from zero; below 2^-126: zero), by integer
+// operations: conversions run on the FP64 pipe.
+__device__ __forceinline__ float near_float(double x) {
+    const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+    const uint32_t mag = hi & 0x7fffffffu;
+    if (mag < 0x38100000u) return 0.0f;
+    uint32_t f = 0x7f800000u;
+    if (mag < 0x47f00000u) f = __funnelshift_l(lo, mag - 0x38000000u, 3) + ((lo >> 28) & 1u);
+    return __uint_as_float((hi & 0x80000000u) | f);
+}
+
 // Bit tests on doubles (integer operations: the FP64 pipe is scarce).
 __device__ __forceinline__ bool dfinite(double x) { return ((__double_as_longlong(x) >> 52) & 0x7ff) != 0x7ff; }
 __device__ __forceinline__ bool dzero(double x) { return (__double_as_longlong(x) << 1) == 0; }
@@ -308,11 +319,12 @@ __device__ __forceinline__ bool dlt0(double x) { return __double_as_longlong(x) 
 // ray in its own pass.  An origin strictly inside the domain (every
 // emission path) needs no clip: the contract's entry time is then 0 and
 // the start point the origin itself.
-template <int KIND>
-__device__ __forceinline__ RayStart ray_setup(const DevGrid &G, const unsigned char *snodes, int n_smem,
-                                              const double *__restrict__ o, const double *__restrict__ d,
-                                              const double *__restrict__ smax, int64_t r, bool estimate = false,
-                                              const float *lat = nullptr) {
+// The descent is locate(p0, p1, p2, sg), the point given by its keys; R.t1 and R.work are estimates that
+// only order and cut the work.
+template <class Locate>
+__device__ __forceinline__ RayStart ray_setup(const DevGrid &G, Locate &&locate, const double *__restrict__ o,
+                                              const double *__restrict__ d, const double *__restrict__ smax,
+                                              int64_t r, bool estimate = false, const float *lat = nullptr) {
     RayStart R;
     R.ik0 = R.ik1 = R.ik2 = 0.0;
     R.ktstart = 0;
@@ -356,8 +368,9 @@ __device__ __forceinline__ RayStart ray_setup(const DevGrid &G, const unsigned c
 #pragma unroll
         for (int a = 0; a < 3; a++)
             if (!dzero(kk[a]))
-                tout = fminf(tout, ((dgt0(kk[a]) ? (float)G.dhi[a] : (float)G.dlo[a]) - (float)oo[a]) / (float)kk[a]);
-        t1f = fminf(tout, (float)tend);
+                tout = fminf(tout, __fdividef((dgt0(kk[a]) ? G.fhi[a] : G.flo[a]) - near_float(oo[a]),
+                                              near_float(kk[a])));
+        t1f = fminf(tout, near_float(tend));
     } else {
         double tout = CUDART_INF;
         int entry = -1;
@@ -393,9 +406,9 @@ __device__ __forceinline__ RayStart ray_setup(const DevGrid &G, const unsigned c
 #pragma unroll
         for (int a = 0; a < 3; a++)
             if (!in_axis(p[a], G.klo[a], G.khi[a], dpos(sg, a), dneg(sg, a), true)) return R;
-        t1f = (float)(tend < tout ? tend : tout);
+        t1f = near_float(tend < tout ? tend : tout);
     }
-    const int32_t c = descend<KIND>(G, snodes, n_smem, p[0], p[1], p[2], sg);
+    const int32_t c = locate(p[0], p[1], p[2], sg);
     if (c < 0) {
         R.sg = HG_RAY_LOST << 8;
         return R;
@@ -408,9 +421,9 @@ __device__ __forceinline__ RayStart ray_setup(const DevGrid &G, const unsigned c
     R.sg = sg;
     R.t1 = t1f;
     if (estimate) {
-        const float of[3] = {(float)oo[0], (float)oo[1], (float)oo[2]};
-        const float kf[3] = {(float)kk[0], (float)kk[1], (float)kk[2]};
-        R.work = work_march(G, lat ? lat : G.work, of, kf, (float)ts, t1f, [](float, float, float, float) {});
+        const float of[3] = {near_float(oo[0]), near_float(oo[1]), near_float(oo[2])};
+        const float kf[3] = {near_float(kk[0]), near_float(kk[1]), near_float(kk[2])};
+        R.work = work_march(G, lat ? lat : G.work, of, kf, near_float(ts), t1f, [](float, float, float, float) {});
     }
     return R;
 }
@@ -719,7 +732,7 @@ struct WalkIO {
     const double *o;
     const double *d;
     const double *smax;
-    const RayStart *starts;
+    const void *starts;  // start records: RayStart (RayStartF on a grid with single-precision bounds)
     double kappa;
     void *tau;
     int32_t *ncross;
@@ -758,6 +771,181 @@ struct WalkIO {
     uint32_t *stg_overflow = nullptr;    // set when the pool ran out
 };
 
+// Sums, counts and outputs of the path or path segment a thread walks.
+//   PREC (MODE_TAU/MODE_FILL): HG_FP64 or HG_FP32K.
+//   PREC (MODE_ADJ): 0 = FP64 gradient atomics, 1 = FP32.
+//   PREC (MODE_TAUADJ): bit 0 the optical depth's (HG_FP32K), bit 1 the gradient's (FP32).
+template <int MODE, int PREC, bool SEGS>
+struct Tally {
+    static constexpr bool STAGE = (MODE == MODE_TAU_STAGE || MODE == MODE_TAUADJ_STAGE);
+    static constexpr bool INTER = (MODE == MODE_INTERACT);
+    static constexpr bool TAU = (MODE == MODE_TAU || MODE == MODE_TAUADJ || STAGE);
+    static constexpr bool ADJ = (MODE == MODE_ADJ || MODE == MODE_TAUADJ || MODE == MODE_TAUADJ_STAGE);
+    static constexpr bool TWO = (MODE == MODE_TAUADJ || MODE == MODE_TAUADJ_STAGE);
+    static constexpr int TPREC = TWO ? (PREC & 1) : (ADJ ? HG_FP64 : PREC);  // HG_FP64 or HG_FP32K
+    static constexpr int GPREC = TWO ? ((PREC >> 1) & 1) : PREC;             // 0 FP64, 1 FP32 gradient
+
+    int64_t ray = 0;      // queue item: a ray, or n_rays + s for path segment s
+    double acc = 0.0;     // FP64 sum of rho*ds
+    float acc32 = 0.0f;   // FP32 Kahan sum
+    float comp32 = 0.0f;  // Kahan compensation
+    int32_t nc = 0;
+    int64_t seg_base = 0;
+    float w32 = 0.0f;
+    double wk = 0.0;  // kappa * w for the adjoint
+    uint32_t st = 0;
+    uint32_t sp = 0;              // staging: next entry position (shifted; 0 = no chunk)
+    double tint = 0.0, it = 0.0;  // interaction: drawn optical depth; interaction time
+    int32_t icell = -1;           // interaction leaf, -1 while none
+    bool walked = false;          // the path has a first leaf (its end time is the current time)
+    float kappa32;
+    unsigned long long keep;
+
+    __device__ __forceinline__ explicit Tally(const WalkIO &io)
+        : kappa32((float)io.kappa), keep(ADJ ? l2_evict_last_policy() : 0ULL) {}
+
+    __device__ __forceinline__ void reset() {
+        acc = 0.0;
+        acc32 = 0.0f;
+        comp32 = 0.0f;
+        nc = 0;
+        st = 0;
+    }
+    // What queue item `ray`, part of ray r, needs beside its geometry.
+    __device__ __forceinline__ void fetch(const WalkIO &io, int64_t r) {
+        if (MODE == MODE_FILL) seg_base = (SEGS && ray >= io.n_rays) ? io.seg_base[ray - io.n_rays] : io.seg_off[r];
+        if (ADJ) w32 = io.w[r];
+        if (INTER) tint = io.tau_int[r];
+    }
+    // Its start; rs as the resume returned it (and returned again).
+    __device__ __forceinline__ int start(const WalkIO &io, int rs) {
+        if (ADJ) wk = io.kappa * (double)w32;
+        if (INTER) {
+            icell = -1;
+            it = 0.0;
+            walked = (rs == WALK_GO);
+            if (((unsigned long long)__double_as_longlong(tint) << 1) > 0xffe0000000000000ULL) {  // NaN
+                st = HG_RAY_BADINPUT;
+                walked = false;
+                rs = WALK_END;
+            }
+        }
+        return rs;
+    }
+    // The crossing of leaf cell: length ds, entered at time key kin, left at tex, density rho (rho32 its
+    // FP32 value, used under FP32K).  Returns true when the walk of the item stops here.
+    __device__ __forceinline__ bool put(const WalkIO &io, int32_t cell, double ds, double rho_leaf, float rho32_leaf,
+                                        long long kin, double tex) {
+        if (INTER) {
+            // stop in the first segment after which kappa * S reaches tau_int; inside it tau grows
+            // linearly: t = t_in + (tau_int - kappa S_before) / (kappa rho), at most the exit time
+            const double s_new = __fma_rn(rho_leaf, ds, acc);
+            if (io.kappa * s_new >= tint) {
+                const double a = tint - io.kappa * acc;
+                const double b = io.kappa * rho_leaf;
+                const double tin = kdouble(kin);
+                double t = tin;
+                if (a > 0.0 && b > 0.0) t = tin + a / b;
+                if (t > tex) t = tex;
+                icell = cell;
+                it = t;
+                nc++;
+                return true;
+            }
+            acc = s_new;
+        }
+        if (TAU) {
+            if (TPREC == HG_FP64) {
+                const double rho = io.rho_ext ? __ldg(io.rho_ext + cell) : rho_leaf;
+                acc = __fma_rn(rho, ds, acc);
+            } else {
+                const float rho32 = io.rho_ext ? __double2float_rn(__ldg(io.rho_ext + cell)) : rho32_leaf;
+                const float kr32 = __fmul_rn(kappa32, rho32);
+                const float y = __fsub_rn(__fmul_rn(kr32, __double2float_rn(ds)), comp32);
+                const float t = __fadd_rn(acc32, y);
+                comp32 = __fsub_rn(__fsub_rn(t, acc32), y);
+                acc32 = t;
+            }
+        }
+        if (MODE == MODE_FILL) {
+            const int64_t idx = seg_base + nc;
+            if (idx >= io.seg_cap) {
+                st |= HG_RAY_OVERFLOW;
+                return true;
+            }
+            io.seg_cell[idx] = cell;
+            if (PREC == HG_FP64)
+                static_cast<double *>(io.seg_ds)[idx] = ds;
+            else
+                static_cast<float *>(io.seg_ds)[idx] = __double2float_rn(ds);
+        }
+        if (STAGE && sp != 0xffffffffu) {
+            if ((sp & (kStageChunk - 1u)) == 0u) {
+                const uint32_t c = (uint32_t)atomicAdd(io.stg_ctr, 1ULL);
+                if (c >= io.stg_nchunks) {
+                    sp = 0xffffffffu;  // pool exhausted: the emission falls back to a fill walk
+                    *io.stg_overflow = 1u;
+                } else {
+                    if (sp != 0u) io.stg_next[((sp - 1u) >> kStageShift) - 1u] = c;
+                    sp = (c + 1u) << kStageShift;
+                }
+            }
+            if (sp != 0xffffffffu) {
+                const uint32_t e = sp - kStageChunk;
+                if (nc == 0) {
+                    if (SEGS && ray >= io.n_rays)
+                        io.stg_start_seg[ray - io.n_rays] = e;
+                    else
+                        io.stg_start_ray[ray] = e;
+                }
+                if (TPREC == HG_FP64)
+                    stage_put(io.stg_ent, e, cell, ds);
+                else
+                    stage_put(io.stg_ent, e, cell, __double2float_rn(ds));
+                sp++;
+            }
+        }
+        if (ADJ) {
+            const double v = wk * ds;
+            const uint32_t slot = ((uint32_t)cell * io.gmul) & io.gmask;
+            if (GPREC == 0)
+                red_add_keep(static_cast<double *>(io.grad) + slot, v, keep);
+            else
+                red_add_keep(static_cast<float *>(io.grad) + slot, __double2float_rn(v), keep);
+        }
+        nc++;
+        return false;
+    }
+    // End of the item in leaf cur at time key ktcur: its outputs.
+    __device__ __forceinline__ void finish(const WalkIO &io, int32_t cur, long long ktcur) {
+        if (SEGS && ray >= io.n_rays) {
+            const int64_t sidx = ray - io.n_rays;
+            if (TAU) {
+                io.part_acc[sidx] = (TPREC == HG_FP64) ? acc : (double)acc32;
+                io.part_nc[sidx] = nc;
+            }
+            io.part_last[sidx] = cur;
+            io.part_st[sidx] = (uint8_t)st;
+        } else if (INTER) {
+            io.int_cell[ray] = icell;
+            io.int_t[ray] = (icell >= 0) ? it : (walked ? kdouble(ktcur) : 0.0);
+            io.ncross[ray] = nc;
+            if (io.status) io.status[ray] = (uint8_t)st;
+        } else if (TAU) {
+            if (TPREC == HG_FP64)
+                static_cast<double *>(io.tau)[ray] = io.kappa * acc;
+            else
+                static_cast<float *>(io.tau)[ray] = acc32;
+            io.ncross[ray] = nc;
+            if (io.status) io.status[ray] = (uint8_t)st;
+        } else if (MODE == MODE_FILL) {
+            if (io.status && st) io.status[ray] |= (uint8_t)st;
+        } else {
+            if (io.status) io.status[ray] = (uint8_t)st;
+        }
+    }
+};
+
 // The walking loop of one thread.  Each iteration loads exactly one leaf
 // record -- the first leaf of a new ray, a listed neighbor to test (the
 // head, or the next tail entry after a miss), or the leaf a top-down
@@ -766,77 +954,41 @@ struct WalkIO {
 // Src hands out rays: bool next(int64_t &ray, const DevGrid *&G, int32_t &max_steps);
 // when Src::kSegments, an item ray >= io.n_rays is path segment
 // ray - io.n_rays of a split ray (otherwise that code is compiled out).
-//   PREC (MODE_TAU/MODE_FILL): HG_FP64 or HG_FP32K.
-//   PREC (MODE_ADJ): 0 = FP64 gradient atomics, 1 = FP32.
-//   PREC (MODE_TAUADJ): bit 0 the optical depth's (HG_FP32K), bit 1 the gradient's (FP32).
+//   PREC: as for Tally.
 //   NAV: 0 the grids hold neighbor lists, 1 ropes, 2 either (read per grid).
 // geo: shared memory for the geometry slots, 9 doubles per thread of the block.
 template <int KIND, int MODE, int PREC, int NAV, class Src>
 __device__ __forceinline__ void walk_loop(Src &src, const WalkIO &io, const unsigned char *snodes, int n_smem,
                                           double *geo) {
     constexpr bool SEGS = Src::kSegments;
-    constexpr bool STAGE = (MODE == MODE_TAU_STAGE || MODE == MODE_TAUADJ_STAGE);
     constexpr bool INTER = (MODE == MODE_INTERACT);
-    constexpr bool TAU = (MODE == MODE_TAU || MODE == MODE_TAUADJ || STAGE);
-    constexpr bool ADJ = (MODE == MODE_ADJ || MODE == MODE_TAUADJ || MODE == MODE_TAUADJ_STAGE);
-    constexpr bool TWO = (MODE == MODE_TAUADJ || MODE == MODE_TAUADJ_STAGE);
-    constexpr int TPREC = TWO ? (PREC & 1) : (ADJ ? HG_FP64 : PREC);  // HG_FP64 or HG_FP32K
-    constexpr int GPREC = TWO ? ((PREC >> 1) & 1) : PREC;             // 0 FP64, 1 FP32 gradient
     const DevGrid *Gp = nullptr;
-    int64_t ray = 0;
     int32_t max_steps = 0;
     RayState S;
     S.g = geo + threadIdx.x;
     S.gs = (int)blockDim.x;
     Leaf L;
     Cand C;
-    double acc = 0.0;     // FP64 sum of rho*ds
-    float acc32 = 0.0f;   // FP32 Kahan sum
-    float comp32 = 0.0f;  // Kahan compensation
-    int32_t nc = 0;
-    int64_t seg_base = 0;
-    double wk = 0.0;  // kappa * w for the adjoint
-    uint32_t st = 0;
+    Tally<MODE, PREC, SEGS> T(io);
     bool have = false;
-    uint32_t sp = 0;  // staging: next entry position (shifted; 0 = no chunk)
-    double tint = 0.0, it = 0.0;  // interaction: drawn optical depth; interaction time
-    int32_t icell = -1;           // interaction leaf, -1 while none
-    bool walked = false;          // the path has a first leaf (its end time is the current time)
-    const float kappa32 = (float)io.kappa;
-    const unsigned long long keep = ADJ ? l2_evict_last_policy() : 0ULL;
     for (;;) {
         if (!have) {
-            if (!src.next(ray, Gp, max_steps)) break;
-            acc = 0.0;
-            acc32 = 0.0f;
-            comp32 = 0.0f;
-            nc = 0;
+            if (!src.next(T.ray, Gp, max_steps)) break;
+            T.reset();
             have = true;
-            int64_t r = ray;
+            int64_t r = T.ray;
             int rs = WALK_GO;
-            st = 0;
-            if (SEGS && ray >= io.n_rays)
-                rs = seg_resume(io.o, io.d, io.smax, io.starts, io.segs, ray - io.n_rays, S, &r);
+            if (SEGS && T.ray >= io.n_rays)
+                rs = seg_resume(io.o, io.d, io.smax, static_cast<const RayStart *>(io.starts), io.segs,
+                                T.ray - io.n_rays, S, &r);
             else
-                rs = ray_resume<SEGS>(io.o, io.d, io.smax, io.starts, ray, S, &st);
+                rs = ray_resume<SEGS>(io.o, io.d, io.smax, static_cast<const RayStart *>(io.starts), T.ray, S, &T.st);
             if (rs == WALK_SKIP) {
                 have = false;
                 continue;
             }
-            if (MODE == MODE_FILL) seg_base = (SEGS && ray >= io.n_rays) ? io.seg_base[ray - io.n_rays] : io.seg_off[r];
-            if (ADJ) wk = io.kappa * (double)io.w[r];
-            if (INTER) {
-                tint = io.tau_int[r];
-                icell = -1;
-                it = 0.0;
-                walked = (rs == WALK_GO);
-                if (((unsigned long long)__double_as_longlong(tint) << 1) > 0xffe0000000000000ULL) {  // NaN
-                    st = HG_RAY_BADINPUT;
-                    walked = false;
-                    rs = WALK_END;
-                }
-            }
-            if (rs == WALK_END) goto finish;
+            T.fetch(io, r);
+            if (T.start(io, rs) == WALK_END) goto finish;
             C.id = S.cur;
             C.mode = CAND_ENTER;
         }
@@ -862,7 +1014,7 @@ __device__ __forceinline__ void walk_loop(Src &src, const WalkIO &io, const unsi
                 }
                 const int32_t j = cand_descend<KIND>(G, snodes, n_smem, S.sg, L, C, start);
                 if (j < 0) {
-                    st = HG_RAY_LOST;
+                    T.st = HG_RAY_LOST;
                     goto finish;
                 }
                 C.id = j;
@@ -874,90 +1026,10 @@ __device__ __forceinline__ void walk_loop(Src &src, const WalkIO &io, const unsi
             bool rec;
             int ax;
             const long long kin = S.ktcur;  // entry time into this leaf
-            const int r = ray_exit<SEGS>(max_steps, S, L, &ds, &rec, &ax, &tex, &st);
+            const int r = ray_exit<SEGS>(max_steps, S, L, &ds, &rec, &ax, &tex, &T.st);
             const bool skip = SEGS && (S.sg & SG_SKIP_FIRST) != 0;  // the segment before records this leaf
             if (SEGS) S.sg &= ~SG_SKIP_FIRST;
-            if (rec && !skip) {
-                if (INTER) {
-                    // stop in the first segment after which kappa * S reaches tau_int; inside it tau grows
-                    // linearly: t = t_in + (tau_int - kappa S_before) / (kappa rho), at most the exit time
-                    const double rho = L.rho;
-                    const double s_new = __fma_rn(rho, ds, acc);
-                    if (io.kappa * s_new >= tint) {
-                        const double a = tint - io.kappa * acc;
-                        const double b = io.kappa * rho;
-                        const double tin = kdouble(kin);
-                        double t = tin;
-                        if (a > 0.0 && b > 0.0) t = tin + a / b;
-                        if (t > tex) t = tex;
-                        icell = S.cur;
-                        it = t;
-                        nc++;
-                        goto finish;
-                    }
-                    acc = s_new;
-                }
-                if (TAU) {
-                    if (TPREC == HG_FP64) {
-                        const double rho = io.rho_ext ? __ldg(io.rho_ext + S.cur) : L.rho;
-                        acc = __fma_rn(rho, ds, acc);
-                    } else {
-                        const float rho32 = io.rho_ext ? __double2float_rn(__ldg(io.rho_ext + S.cur)) : L.rho32;
-                        const float kr32 = __fmul_rn(kappa32, rho32);
-                        const float y = __fsub_rn(__fmul_rn(kr32, __double2float_rn(ds)), comp32);
-                        const float t = __fadd_rn(acc32, y);
-                        comp32 = __fsub_rn(__fsub_rn(t, acc32), y);
-                        acc32 = t;
-                    }
-                }
-                if (MODE == MODE_FILL) {
-                    const int64_t idx = seg_base + nc;
-                    if (idx >= io.seg_cap) {
-                        st |= HG_RAY_OVERFLOW;
-                        goto finish;
-                    }
-                    io.seg_cell[idx] = S.cur;
-                    if (PREC == HG_FP64)
-                        static_cast<double *>(io.seg_ds)[idx] = ds;
-                    else
-                        static_cast<float *>(io.seg_ds)[idx] = __double2float_rn(ds);
-                }
-                if (STAGE && sp != 0xffffffffu) {
-                    if ((sp & (kStageChunk - 1u)) == 0u) {
-                        const uint32_t c = (uint32_t)atomicAdd(io.stg_ctr, 1ULL);
-                        if (c >= io.stg_nchunks) {
-                            sp = 0xffffffffu;  // pool exhausted: the emission falls back to a fill walk
-                            *io.stg_overflow = 1u;
-                        } else {
-                            if (sp != 0u) io.stg_next[((sp - 1u) >> kStageShift) - 1u] = c;
-                            sp = (c + 1u) << kStageShift;
-                        }
-                    }
-                    if (sp != 0xffffffffu) {
-                        const uint32_t e = sp - kStageChunk;
-                        if (nc == 0) {
-                            if (SEGS && ray >= io.n_rays)
-                                io.stg_start_seg[ray - io.n_rays] = e;
-                            else
-                                io.stg_start_ray[ray] = e;
-                        }
-                        if (TPREC == HG_FP64)
-                            stage_put(io.stg_ent, e, S.cur, ds);
-                        else
-                            stage_put(io.stg_ent, e, S.cur, __double2float_rn(ds));
-                        sp++;
-                    }
-                }
-                if (ADJ) {
-                    const double v = wk * ds;
-                    const uint32_t slot = ((uint32_t)S.cur * io.gmul) & io.gmask;
-                    if (GPREC == 0)
-                        red_add_keep(static_cast<double *>(io.grad) + slot, v, keep);
-                    else
-                        red_add_keep(static_cast<float *>(io.grad) + slot, __double2float_rn(v), keep);
-                }
-                nc++;
-            }
+            if (rec && !skip && T.put(io, S.cur, ds, L.rho, L.rho32, kin, tex)) goto finish;
             if (r == WALK_GO) {
                 if (NAV == 0 || (NAV == 2 && G.nav == HG_NAV_NEIGHBOR_LISTS))
                     cand_first<0, INTER>(S, L, ax, tex, C);
@@ -967,7 +1039,7 @@ __device__ __forceinline__ void walk_loop(Src &src, const WalkIO &io, const unsi
                     C.id = rope_descend<KIND>(G, snodes, n_smem, S.sg, L.lo(ax), L.hi(ax), C);
                     C.mode = CAND_TEST;
                     if (C.id < 0) {
-                        st = HG_RAY_LOST;
+                        T.st = HG_RAY_LOST;
                         goto finish;
                     }
                 }
@@ -975,31 +1047,7 @@ __device__ __forceinline__ void walk_loop(Src &src, const WalkIO &io, const unsi
             }
         }
     finish:
-        if (SEGS && ray >= io.n_rays) {
-            const int64_t sidx = ray - io.n_rays;
-            if (TAU) {
-                io.part_acc[sidx] = (TPREC == HG_FP64) ? acc : (double)acc32;
-                io.part_nc[sidx] = nc;
-            }
-            io.part_last[sidx] = S.cur;
-            io.part_st[sidx] = (uint8_t)st;
-        } else if (INTER) {
-            io.int_cell[ray] = icell;
-            io.int_t[ray] = (icell >= 0) ? it : (walked ? kdouble(S.ktcur) : 0.0);
-            io.ncross[ray] = nc;
-            if (io.status) io.status[ray] = (uint8_t)st;
-        } else if (TAU) {
-            if (TPREC == HG_FP64)
-                static_cast<double *>(io.tau)[ray] = io.kappa * acc;
-            else
-                static_cast<float *>(io.tau)[ray] = acc32;
-            io.ncross[ray] = nc;
-            if (io.status) io.status[ray] = (uint8_t)st;
-        } else if (MODE == MODE_FILL) {
-            if (io.status && st) io.status[ray] |= (uint8_t)st;
-        } else {
-            if (io.status) io.status[ray] = (uint8_t)st;
-        }
+        T.finish(io, S.cur, S.ktcur);
         have = false;
     }
 }
