@@ -232,7 +232,7 @@ hg_status load_grid_impl(const hg_grid_desc *desc, const int32_t *ropes, int32_t
 // Whether every node bound is a single-precision number of the range that the single-precision records and
 // walks are made for (LeafRecF), and the links fit the nodes' fields.
 bool single_precision_bounds(const hg_grid_desc &D) {
-    if (D.n_nodes >= (1 << 29)) return false;
+    if (D.n_nodes >= (1 << 29) || D.n_leaves >= (1 << hg::kStepShift)) return false;
     double most = 0.0;
     for (int a = 0; a < 3; a++) most = std::max(most, std::max(std::fabs(D.node_lo[a]), std::fabs(D.node_hi[a])));
     if (!(most >= 0x1p-20 && most <= 0x1p20)) return false;
@@ -245,16 +245,13 @@ bool single_precision_bounds(const hg_grid_desc &D) {
     return true;
 }
 
-// Wall w of a leaf in its single-precision record: *first and the step bits (LeafRecF) from the wall's
-// neighbor list.
-uint32_t wall_slot(const hg_grid_desc &D, const std::vector<int64_t> &leaf_node, const std::vector<int32_t> &parent,
-                   int64_t leaf, int w, int32_t *first) {
+// Wall w of a leaf in its single-precision record (LeafRecF), from the wall's neighbor list.
+int32_t wall_slot(const hg_grid_desc &D, const std::vector<int64_t> &leaf_node, const std::vector<int32_t> &parent,
+                  int64_t leaf, int w) {
     const int64_t b0 = D.nbr_off[6 * leaf + w], cnt = D.nbr_off[6 * leaf + w + 1] - b0;
     const int32_t *nb = D.nbr_id + b0;
-    *first = -1;
-    if (cnt <= 0) return 0;
-    *first = nb[0];
-    if (cnt == 1) return 0;
+    if (cnt <= 0) return -1;
+    if (cnt == 1) return nb[0];
     const int a = w >> 1, s = w & 1;
     const int ax[2] = {a == 0 ? 1 : 0, a == 2 ? 1 : 2};
     const double *flo = D.node_lo + 3 * leaf_node[(size_t)leaf], *fhi = D.node_hi + 3 * leaf_node[(size_t)leaf];
@@ -286,17 +283,13 @@ uint32_t wall_slot(const hg_grid_desc &D, const std::vector<int64_t> &leaf_node,
             bits |= (step == 1 ? 1u : step == 2 ? 2u : 3u) << (2 * b);
         }
         if (ok && cnt == 4) ok = at[3] == at[1] + at[2] - at[0];
-        if (ok) {
-            *first = at[0];
-            return bits << (4 * w);
-        }
+        if (ok) return at[0] | (int32_t)(bits << hg::kStepShift);
     }
     // the rope node: the first ancestor of a neighbor that covers the face
     const double P = s ? fhi[a] : flo[a];
     int64_t nd = leaf_node[(size_t)nb[0]];
     while (nd > 0 && !rope_covers(D, nd, a, s, P, flo, fhi)) nd = parent[(size_t)nd];
-    *first = (int32_t)(-2 - nd);
-    return 0;
+    return (int32_t)(-2 - nd);
 }
 
 }  // namespace
@@ -519,12 +512,12 @@ hg_status load_grid_impl(const hg_grid_desc *desc, const int32_t *ropes, int32_t
                         }
                         R.rho = D.leaf_rho[i];
                         R.rho32 = (float)D.leaf_rho[i];
-                        R.steps = 0;
+                        R.pad = 0;
                         for (int w = 0; w < 6; w++) {
                             if (ropes) {
                                 R.first[w] = ropes[6 * i + w];
                             } else {
-                                R.steps |= wall_slot(D, leaf_node, parent, i, w, &R.first[w]);
+                                R.first[w] = wall_slot(D, leaf_node, parent, i, w);
                                 many += D.nbr_off[6 * i + w + 1] - D.nbr_off[6 * i + w] > kScanLimit;
                             }
                         }

@@ -71,11 +71,11 @@ static_assert(sizeof(KdNode) == 16 && sizeof(OctNode) == 32, "node sizes");
 // one 64-byte DRAM access, where a 96-byte record always takes two -- and the walks decide most
 // crossings in single precision (walkf.cuh).  Grids with other bounds keep the records above.
 //   sector 0: lo.x lo.y lo.z hi.x hi.y hi.z (f32) rho
-//   sector 1: first[6] rho32 steps
+//   sector 1: first[6] rho32 pad
 // first[w]: -1 when wall w lies on the domain boundary; the neighbor when one leaf covers the wall's face;
-// with steps bits 4w .. 4w+3 (e1 | e2 << 2) not zero, the leaf at the lower corner of the face, which two
-// or four equal leaves share, the leaf in the upper half on the first (second) of the two other axes
-// having an id higher by 2^(e1-1) (2^(e2-1)); otherwise -2 - the wall's rope node, the deepest node across
+// when two or four equal leaves share the face, the leaf at its lower corner, with e1 | e2 << 2 in the bits
+// from kStepShift: the leaf in the upper half on the first (second) of the two other axes has an id higher
+// by 2^(e1-1) (2^(e2-1)), e = 0 where the axis is not halved; otherwise -2 - the wall's rope node, the deepest node across
 // it that covers the face.  With HG_NAV_ROPES every wall of more than one neighbor holds its rope.
 struct alignas(32) LeafRecF {
     float lo[3];
@@ -83,8 +83,9 @@ struct alignas(32) LeafRecF {
     double rho;
     int32_t first[6];
     float rho32;
-    uint32_t steps;
+    uint32_t pad;
 };
+constexpr int kStepShift = 27;  // (LeafRecF) leaf ids are smaller than 2^27
 static_assert(sizeof(LeafRecF) == 64, "single-precision leaf record must be two sectors");
 
 // link = first child << 2 | split axis, or leaf << 2 | 3.

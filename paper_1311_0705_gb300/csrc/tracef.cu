@@ -7,9 +7,11 @@
 
 namespace hg {
 
-// As trace_kernel (trace.cu), either tree and navigation.
+// As trace_kernel (trace.cu), either tree and navigation.  Four blocks of 256 threads per SM at 64 registers;
+// the interaction search, which carries the drawn depth and its own state, spills 72 bytes there and runs
+// with three blocks at 80 (1e6 packets, disk octree: call 747 -> 687 us).
 template <int MODE, int PREC>
-__global__ void __launch_bounds__(256, 4) trace_kernel_f(const __grid_constant__ TraceArgs A) {
+__global__ void __launch_bounds__(256, MODE == MODE_INTERACT ? 3 : 4) trace_kernel_f(const __grid_constant__ TraceArgs A) {
     extern __shared__ __align__(16) unsigned char smem[];
     if (A.run_if && *A.run_if == 0u) return;  // a fallback walk with nothing to do
     GridRays src(A);

@@ -61,8 +61,12 @@
 // Measured, 1e6 rays on the disk octree, FP64 optical depth: the walk of walk.cuh 969 us; these records
 // and decisions inside its loop 960 us (the refill -- queue atomic, order, start record, first leaf -- and
 // the searches are chains of dependent loads that every round of a warp waits for: issue slots 38 % used,
-// 16 of 32 lanes active); with the lane states 598 us (59 %, 20 lanes).  DRAM reads 2.3 -> 1.1 GB.  FP64
-// pipe 46 % busy: its 4 operations per crossing bound the walk at 235 us.
+// 16 of 32 lanes active); with the lane states 598 us (59 %, 20 lanes; L1 wavefronts 57-62 %).  DRAM reads
+// 2.3 -> 1.1 GB.  FP64 pipe 46 % busy: its 4 operations per crossing bound the walk at 235 us.  What is left is
+// instructions, so they are few: the steps to equal neighbors in the spare bits of the wall slot, one comparison of
+// the high words for "later than now, before the end" (the rest in the branch not taken), the two parts of eps in
+// shared memory, and no register spills in the optical-depth walk (20 bytes of them cost it 12 %): calls
+// 905 -> 797 us (1e6 rays, disk octree), 12.88 -> 11.57 ms (1e7, torus, FP32K).
 #pragma once
 
 #include "walk.cuh"
@@ -201,27 +205,28 @@ struct RawRec {
     __device__ __forceinline__ double rho() const { return d(6); }
     __device__ __forceinline__ int32_t first(int w) const { return (int32_t)v[8 + w]; }
     __device__ __forceinline__ float rho32() const { return __uint_as_float(v[14]); }
-    __device__ __forceinline__ uint32_t steps() const { return v[15]; }
 };
 
 // Per-ray walking state.  Shared memory holds, per thread, {o32, i32, E, k32} of each axis and the origin
-// and 1/d in FP64 (96 bytes; slots strided by the block so that a warp's accesses fall on consecutive
-// words): with them in registers four 256-thread blocks would not fit on an SM.
-constexpr int kGeoBytesF = 96;
+// and 1/d in FP64, and the two parts of eps (104 bytes; slots strided by the block so that a warp's accesses
+// fall on consecutive words): with them in registers four 256-thread blocks would not fit on an SM.
+constexpr int kGeoBytesF = 104;
 struct RayStateF {
     float4 *a;  // this thread's first axis slot
     double *g;  // its first FP64 slot
+    float2 *e;  // {slope, constant} of eps in the width of the exit time's bounds
     int gs;     // slot stride
     long long ktcur;   // key of the current time
-    long long klim;    // smaller of the keys of the path's end and of the time a path segment stops after
+    long long klim;    // smaller of the keys of the path's end and of the time a path segment stops after;
+                       // -1 while the segment's first leaf, which the segment before records, is walked
     float tp;          // upper bound of the current time
-    float base;        // the constant part of eps
     uint32_t sg;
     int32_t cur, steps;  // current leaf; steps left
     __device__ __forceinline__ void bind(unsigned char *geo) {
         gs = (int)blockDim.x;
         a = reinterpret_cast<float4 *>(geo) + threadIdx.x;
         g = reinterpret_cast<double *>(geo + (size_t)gs * 3 * sizeof(float4)) + threadIdx.x;
+        e = reinterpret_cast<float2 *>(geo + (size_t)gs * (3 * sizeof(float4) + 6 * sizeof(double))) + threadIdx.x;
     }
     __device__ __forceinline__ double o(int x) const { return g[x * gs]; }
     __device__ __forceinline__ double ik(int x) const { return g[(3 + x) * gs]; }
@@ -230,13 +235,13 @@ struct RayStateF {
 // Geometry of a ray from its start record (SG_EXACT rays: E and base infinite, the rest of no account).
 __device__ __forceinline__ void start_geometry(const RawRec &V, float fdom, RayStateF &S) {
     const bool exact = (V.v[15] & SG_EXACT) != 0;
-    float o32[3], scale = 0.0f;
+    float o32[3], scale = 0.0f, kmax = 0.0f;
 #pragma unroll
     for (int x = 0; x < 3; x++) {
         o32[x] = near_float(V.d(8 + 2 * x));
         scale = fmaxf(scale, fabsf(o32[x]));
     }
-    S.base = exact ? CUDART_INF_F : 4.5f * 0x1p-24f * (scale + fdom);
+    const float base = exact ? CUDART_INF_F : 4.5f * 0x1p-24f * (scale + fdom);
 #pragma unroll
     for (int x = 0; x < 3; x++) {
         const double ik = V.d(2 * x);
@@ -247,12 +252,14 @@ __device__ __forceinline__ void start_geometry(const RawRec &V, float fdom, RayS
         if (i32 == 0.0f) {
             i32 = 0x1p100f;
             k32 = 0.0f;
-            e = 0x1p100f * S.base;
+            e = 0x1p100f * base;
         }
+        kmax = fmaxf(kmax, fabsf(k32));
         S.a[x * S.gs] = make_float4(o32[x], i32, exact ? CUDART_INF_F : e, k32);
         S.g[x * S.gs] = V.d(8 + 2 * x);
         S.g[(3 + x) * S.gs] = ik;
     }
+    S.e[0] = make_float2(0.501f * kmax, base);
 }
 
 // The exit wall by the contract's FP64 arithmetic: smallest time, ties to the lower axis (-1: no wall in finite time).
@@ -321,7 +328,8 @@ __device__ __forceinline__ bool locate_step(const DevGrid &G, const WalkIO &io, 
     const int ax = C.ax & 3;
     const float e = (C.ax & CAND_EXACT) ? -1.0f : C.eps;
     // a point on the wall belongs to the side the ray goes to
-    const float fw = dir_float(widen(C.wall), dneg(S.sg, ax));
+    const bool neg = dneg(S.sg, ax);
+    auto upper = [&](int x, float p, float s) { return x != ax ? p >= s : (neg ? C.wall > s : C.wall >= s); };
     bool open;
     int32_t next;
     if (G.kind == HG_KDTREE) {
@@ -333,9 +341,9 @@ __device__ __forceinline__ bool locate_step(const DevGrid &G, const WalkIO &io, 
             return true;
         }
         const float s = __uint_as_float(V.v[0]);
-        const float p = x == ax ? fw : (x == (ax == 0 ? 1 : 0) ? C.p1 : C.p2);
+        const float p = x == (ax == 0 ? 1 : 0) ? C.p1 : C.p2;
         open = x != ax && !(fabsf(p - s) > e);
-        next += p >= s ? 1 : 0;
+        next += upper(x, p, s) ? 1 : 0;
     } else {
         const int32_t link = (int32_t)V.v[3];
         if (link < 0) {
@@ -343,9 +351,9 @@ __device__ __forceinline__ bool locate_step(const DevGrid &G, const WalkIO &io, 
             return true;
         }
         const float s0 = __uint_as_float(V.v[0]), s1 = __uint_as_float(V.v[1]), s2 = __uint_as_float(V.v[2]);
-        const float p0 = ax == 0 ? fw : C.p1, p1 = ax == 1 ? fw : (ax == 0 ? C.p1 : C.p2), p2 = ax == 2 ? fw : C.p2;
+        const float p0 = C.p1, p1 = ax == 0 ? C.p1 : C.p2, p2 = C.p2;
         open = !((ax == 0 || fabsf(p0 - s0) > e) && (ax == 1 || fabsf(p1 - s1) > e) && (ax == 2 || fabsf(p2 - s2) > e));
-        next = link + (p0 >= s0 ? 1 : 0) + (p1 >= s1 ? 2 : 0) + (p2 >= s2 ? 4 : 0);
+        next = link + (upper(0, p0, s0) ? 1 : 0) + (upper(1, p1, s1) ? 2 : 0) + (upper(2, p2, s2) ? 4 : 0);
     }
     if (open) {
         exit_point_exact(G, io, r, S, C);
@@ -360,8 +368,9 @@ __device__ __forceinline__ bool locate_step(const DevGrid &G, const WalkIO &io, 
 // queue is empty.
 enum { LANE_WALK = 0, LANE_START = 1, LANE_NODE = 2, LANE_DONE = 3, LANE_EXIT = 4 };
 // Idle lanes of a warp that are refilled together: a refill is ~100 instructions whatever the number of
-// lanes taking part, an idle lane costs its share of a round.
-constexpr int kRefill = 4;
+// lanes taking part, an idle lane costs its share of a round.  2, 4, 6, 8 lanes: disk octree (1e6 rays) 887,
+// 873, 867, 858 us, torus (1e7) 11.62, 11.48, 11.67, 11.90 ms per call.
+constexpr int kRefill = 5;
 struct PoolItem {
     int64_t item;  // queue item: a ray, or n_rays + s for path segment s
     int64_t of;    // the ray it is, or is part of (batches: its grid)
@@ -453,12 +462,13 @@ __device__ __forceinline__ void walk_loop_f(Src &src, const WalkIO &io, unsigned
                 if (!(q > C.eps)) {  // not certainly inside
                     if (!(C.ax & CAND_EXACT)) exit_point_exact(G, io, ray_of(), S, C);
                     if (!(l1 <= C.p1 && C.p1 < h1 && l2 <= C.p2 && C.p2 < h2)) {
-                        // an exit point on the domain surface with the direction pointing out ends the path
+                        // an exit point on the domain surface with the direction pointing out ends the path;
+                        // else it is on an edge or corner: located from the root
                         const float gl1 = x0 ? G.flo[1] : G.flo[0], gh1 = x0 ? G.fhi[1] : G.fhi[0];
                         const float gl2 = x2 ? G.flo[1] : G.flo[2], gh2 = x2 ? G.fhi[1] : G.fhi[2];
                         if (!(gl1 <= C.p1 && C.p1 < gh1 && gl2 <= C.p2 && C.p2 < gh2)) {
                             state = LANE_DONE;
-                        } else {  // edge or corner exit: locate the exit point from the root
+                        } else {
                             C.left = (G.max_depth + 1) | CAND_ROOT;
                             C.id = 0;
                             V.load_node(G, 0);
@@ -469,14 +479,9 @@ __device__ __forceinline__ void walk_loop_f(Src &src, const WalkIO &io, unsigned
                 }
             }
             S.cur = C.id;
-            if (S.steps <= 0) {
-                T.st = HG_RAY_STEPLIMIT;
-                state = LANE_DONE;
-                goto next_round;
-            }
-            S.steps--;
             // exit wall
             const float4 A0 = S.a[0], A1 = S.a[S.gs], A2 = S.a[2 * S.gs];  // {o32, i32, E, k32}
+            const float2 ep = S.e[0];
             const float w0 = dneg(sg, 0) ? V.lo(0) : V.hi(0);
             const float w1 = dneg(sg, 1) ? V.lo(1) : V.hi(1);
             const float w2 = dneg(sg, 2) ? V.lo(2) : V.hi(2);
@@ -490,9 +495,11 @@ __device__ __forceinline__ void walk_loop_f(Src &src, const WalkIO &io, unsigned
             const bool q0 = !(tl0 > m), q1 = !(tl1 > m), q2 = !(tl2 > m);
             const bool sure = ((q0 != q1) != q2) && !(q0 && q1) && m >= S.tp;  // exactly one
             int ax = q0 ? 0 : (q1 ? 1 : 2);
-            long long kt = KEY_INF;
+            bool nowall = false;
             if (!sure) {
+                long long kt;
                 ax = exit_exact(S, V, &kt);
+                nowall = ax < 0;
                 ml = floor_float(kdouble(kt < S.ktcur ? S.ktcur : kt));
                 m = __fmaf_rn(ml, 1.0f + 0x1p-21f, 0x1p-126f);
             }
@@ -501,27 +508,28 @@ __device__ __forceinline__ void walk_loop_f(Src &src, const WalkIO &io, unsigned
             const int32_t g0 = dneg(sg, 0) ? V.first(0) : V.first(1);
             const int32_t g1 = dneg(sg, 1) ? V.first(2) : V.first(3);
             const int32_t g2 = dneg(sg, 2) ? V.first(4) : V.first(5);
-            int32_t f = ax < 0 ? -1 : (x0 ? g0 : (x1 ? g1 : g2));
+            int32_t f = x0 ? g0 : (x1 ? g1 : g2);
             // exit point
             const float wid = m - ml;
             const float tm = __fmaf_rn(-0.5f, wid, m);
-            C.eps = __fmaf_rn(0.501f * fmaxf(fmaxf(fabsf(A0.w), fabsf(A1.w)), fabsf(A2.w)), wid, S.base);
+            C.eps = __fmaf_rn(ep.x, wid, ep.y);
             const float p0 = __fmaf_rn(A0.w, tm, A0.x), p1 = __fmaf_rn(A1.w, tm, A1.x), p2 = __fmaf_rn(A2.w, tm, A2.x);
             C.p1 = x0 ? p1 : p0;
             C.p2 = (x0 || x1) ? p2 : p1;
             C.ax = ax;
             S.tp = m;
-            // which of two or four equal neighbors
-            const uint32_t steps = f >= 0 ? (V.steps() >> (8 * ax + (dneg(sg, ax) ? 0 : 4))) & 15u : 0u;
-            if (steps) {
+            if (f >= 1 << kStepShift) {  // which of two or four equal neighbors
+                const uint32_t steps = (uint32_t)f >> kStepShift;
                 const bool x2 = ax == 2;
                 const float m1 = 0.5f * (x0 ? V.lo(1) + V.hi(1) : V.lo(0) + V.hi(0));
                 const float m2 = 0.5f * (x2 ? V.lo(1) + V.hi(1) : V.lo(2) + V.hi(2));
+                f &= (1 << kStepShift) - 1;
                 f += C.p1 >= m1 ? (1 << (steps & 3u)) >> 1 : 0;
                 f += C.p2 >= m2 ? (1 << (steps >> 2)) >> 1 : 0;
             }
             const double rho = V.rho();
             const float rho32 = USE32 ? V.rho32() : 0.0f;
+            if (nowall) f = -1;
             if (f >= 0) {
                 C.id = f;
                 V.load(records() + f);
@@ -532,23 +540,35 @@ __device__ __forceinline__ void walk_loop_f(Src &src, const WalkIO &io, unsigned
                 state = LANE_NODE;
             }
             // the exit time, the segment and its sums, while the next record is under way
-            if (sure) kt = __double_as_longlong((widen(C.wall) - S.o(ax)) * S.ik(ax));
-            bool end = f == -1;
+            long long kt = KEY_INF;
+            if (!nowall) kt = __double_as_longlong((widen(C.wall) - S.o(ax)) * S.ik(ax));
+            bool end = f == -1, put = true;
             const long long kin = S.ktcur;
-            if (kt > S.klim) {  // the path or its segment ends here
+            const int hi = (int)(kt >> 32);
+            S.steps--;
+            if (!(hi > (int)(kin >> 32) && hi < (int)(S.klim >> 32) && S.steps >= 0)) {
+                // no later than the current time, or near or past the end of the path, its segment or its steps
                 const bool seg = SEGS && T.ray >= io.n_rays;
                 const long long ktend = io.smax ? okey(io.smax[ray_of()]) : KEY_INF;
-                end = end || (seg && kt > io.segs[T.ray - io.n_rays].ktstop);
+                const long long ktstop = seg ? io.segs[T.ray - io.n_rays].ktstop : KEY_INF;
+                const bool skip = SEGS && S.klim < 0;  // the segment before records this leaf
+                S.klim = ktend < ktstop ? ktend : ktstop;
                 if (ktend < kt) {
                     kt = ktend;
                     end = true;
                 }
+                if (kt < kin) kt = kin;
+                end = end || (SEGS && kt > ktstop);
+                put = kt != kin && !skip;
+                if (S.steps < 0) {
+                    T.st = HG_RAY_STEPLIMIT;
+                    kt = kin;
+                    end = true;
+                    put = false;
+                }
             }
-            if (kt < kin) kt = kin;
             S.ktcur = kt;
-            const bool skip = SEGS && (sg & SG_SKIP_FIRST) != 0;  // the segment before records this leaf
-            if (SEGS) S.sg = sg & ~SG_SKIP_FIRST;
-            if (kt != kin && !skip) {
+            if (put) {
                 const double tex = __longlong_as_double(kt);
                 if (T.put(io, S.cur, tex - __longlong_as_double(kin), rho, rho32, kin, tex)) end = true;
             }
@@ -566,8 +586,9 @@ __device__ __forceinline__ void walk_loop_f(Src &src, const WalkIO &io, unsigned
             } else if (rs == WALK_GO) {
                 const long long ktend = okey(__longlong_as_double(S.ktcur));
                 if (ktend < S.klim) S.klim = ktend;
+                if (SEGS && (sg & SG_SKIP_FIRST)) S.klim = -1;
                 start_geometry(V, grid().fdom, S);
-                S.sg = sg & 0xffu;
+                S.sg = sg & 0x3fu;
                 S.ktcur = (long long)(((unsigned long long)V.v[7] << 32) | V.v[6]);
                 S.tp = __fmaf_rn(floor_float(__longlong_as_double(S.ktcur)), 1.0f + 0x1p-21f, 0x1p-126f);
                 if (S.ktcur == 0) S.tp = 0.0f;
