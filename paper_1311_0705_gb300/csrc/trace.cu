@@ -21,8 +21,8 @@ namespace hg {
 // Crossings per path are heavy-tailed (on the disk grids the median path
 // crosses 5 leaves, the longest several hundred), and a launch lasts at
 // least as long as its longest path.  So with a non-NULL bucket_count the
-// pass also sorts the rays into kBuckets classes of estimated work (the
-// coarse-lattice estimate, or the exact count when seg_off gives it) and
+// pass also counts the rays in kBuckets classes of estimated work (the
+// coarse-lattice estimate, or the exact count when seg_off gives it), and
 // the dynamic queue hands out the heaviest paths first.
 constexpr int kBuckets = 32;
 
@@ -40,8 +40,8 @@ __device__ __forceinline__ int work_bucket(float w) {
 // With a non-NULL work_total the pass also adds up the rays' estimated work
 // (each rounded up to an integer, so the total does not depend on the order
 // of the additions); the split planner sizes path segments from it.
-// F: the grid holds single-precision records; the start records are then RayStartF and t1, when not NULL,
-// receives the ends of the estimates' marches.
+// work and t1, when not NULL, receive the estimates and the ends of the intervals they cover.
+// F: the grid holds single-precision records; the start records are then RayStartF.
 template <int KIND, bool F>
 __global__ void __launch_bounds__(256) setup_kernel(const DevGrid G, int64_t n, const double *__restrict__ o,
                                                     const double *__restrict__ d, const double *__restrict__ smax,
@@ -53,7 +53,7 @@ __global__ void __launch_bounds__(256) setup_kernel(const DevGrid G, int64_t n, 
     if (threadIdx.x < kBuckets) hist[threadIdx.x] = 0;
     const int node_bytes = n_smem * node_size<KIND, F>();
     // the work lattice follows the staged nodes when the pass estimates work
-    const bool estimate = bucket_count != nullptr && !seg_off;
+    const bool estimate = work != nullptr && !seg_off;
     float *lat = (estimate && G.work) ? reinterpret_cast<float *>(smem + geo_offset(node_bytes)) : nullptr;
     if (lat) stage_lattice(G, lat);
     stage_nodes(G.nodes, node_bytes, smem);
@@ -65,17 +65,17 @@ __global__ void __launch_bounds__(256) setup_kernel(const DevGrid G, int64_t n, 
                 return F ? locate_key_f<KIND>(G, smem, n_smem, p0, p1, p2, sg)
                          : descend<KIND>(G, smem, n_smem, p0, p1, p2, sg);
             },
-            o, d, smax, r, estimate, lat);
+            o, d, smax, r, lat);
         if (seg_off) R.work = (float)(seg_off[r + 1] - seg_off[r]);
         if (F) {
             static_cast<RayStartF *>(starts)[r] = start_f(R, o, d, r);
-            if (t1) t1[r] = R.t1;
         } else {
             static_cast<RayStart *>(starts)[r] = R;
         }
         if (work) work[r] = R.work;
+        if (t1) t1[r] = R.t1;
         if (bucket_count) atomicAdd(&hist[work_bucket(R.work)], 1u);
-        wsum += (unsigned long long)ceilf(fmaxf(R.work, 0.0f));
+        wsum += (unsigned long long)__float2uint_ru(fmaxf(R.work, 0.0f));
     }
     if (work_total) {
         for (int off = 16; off > 0; off >>= 1) wsum += __shfl_down_sync(0xffffffffu, wsum, off);
@@ -126,28 +126,25 @@ struct SplitRec {
 // (only those can outlast the launch's bulk when the heaviest go first),
 // into K = min(16, ceil(w / W)) pieces of equal estimated work,
 // W = max(32, A / 2).  Forced: every ray of more than 3 estimated crossings,
-// W = 2.  One warp per ray, over the heavy end of the work-ordered queue:
-// the lanes sample the work lattice at 32 points of the path and sum them
-// (a warp prefix sum), lane j places cut j where the sum reaches (j + 1) / K
+// W = 2.  Half a warp per ray (a ray has at most 15 cuts), over the heavy
+// end of the work-ordered queue, or over all rays when there is none: the
+// lanes sample the work lattice at 32 points of the path and sum them
+// (a prefix sum), lane j places cut j where the sum reaches (j + 1) / K
 // of the total (descent and depth test), and the accepted cuts are those of
 // increasing t_c in distinct leaves, in path order.  Segment slots are
 // taken with one atomic per ray; their count is bounded (sum over split
 // rays of ceil(w/W) <= total/W + total/max(64, A) <= 3 T, or 16 n when
 // forced), so seg_cap is never reached -- if it were, the ray would stay
 // whole and the slots taken would be marked empty.
-constexpr int kPlanWarps = 8;  // warps per 256-thread block
+// A ray's chain of dependent loads (queue, start record, one per tree level,
+// leaf) is what the pass waits for: with a warp per ray, half of its lanes idle
+// in the descents, 1e6 rays on the disk octree took 52 us, now 45 (k-d 62, now 43).
+constexpr int kPlanRays = 16;  // rays per 256-thread block at a time
 
-__device__ __forceinline__ float start_work(const RayStart &R, const float *, int64_t) { return R.work; }
-__device__ __forceinline__ float start_work(const RayStartF &, const float *work, int64_t r) { return work[r]; }
-__device__ __forceinline__ float start_t1(const RayStart &R, const float *, int64_t) { return R.t1; }
-__device__ __forceinline__ float start_t1(const RayStartF &, const float *t1, int64_t r) { return t1[r]; }
-
-// F: single-precision records (the work estimates and march ends come from work and t1).
 template <int KIND, bool F>
 __global__ void __launch_bounds__(256) split_kernel(const DevGrid G, int64_t n, const double *__restrict__ o,
-                                                    const double *__restrict__ d, const double *__restrict__ smax,
-                                                    void *starts_v, const float *__restrict__ work,
-                                                    const float *__restrict__ t1,
+                                                    const double *__restrict__ d, void *starts_v,
+                                                    const float *__restrict__ work, const float *__restrict__ t1,
                                                     const unsigned long long *work_total,
                                                     const unsigned long long *bucket_count,
                                                     const int64_t *__restrict__ order, int64_t threads, int force,
@@ -155,8 +152,8 @@ __global__ void __launch_bounds__(256) split_kernel(const DevGrid G, int64_t n, 
                                                     SplitRec *list, unsigned long long *split_count) {
     using Start = typename std::conditional<F, RayStartF, RayStart>::type;
     Start *starts = static_cast<Start *>(starts_v);
-    __shared__ int32_t s_leaf[kPlanWarps][kMaxSegs];
-    __shared__ long long s_key[kPlanWarps][kMaxSegs];
+    __shared__ int32_t s_leaf[kPlanRays][kMaxSegs];
+    __shared__ long long s_key[kPlanRays][kMaxSegs];
     __shared__ long long s_ncand;
     __shared__ __align__(16) float lat[kWorkN * kWorkN * kWorkN];
     if (!G.work || G.work_n <= 0) return;
@@ -166,71 +163,80 @@ __global__ void __launch_bounds__(256) split_kernel(const DevGrid G, int64_t n, 
     const float thr = force ? 3.0f : fmaxf(64.0f, A);
     if (threadIdx.x == 0) {
         // the queue is sorted by work bucket: candidates are the buckets up to that of the threshold
-        const int bt = work_bucket(thr);
-        long long c = 0;
-        for (int b = 0; b <= bt; b++) c += (long long)bucket_count[b];
+        long long c = n;
+        if (order) {
+            const int bt = work_bucket(thr);
+            c = 0;
+            for (int b = 0; b <= bt; b++) c += (long long)bucket_count[b];
+        }
         s_ncand = c;
     }
     __syncthreads();
     const long long ncand = s_ncand;
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
+    const int lane = threadIdx.x & 15, slot = threadIdx.x >> 4;  // lane of the half warp, ray slot in the block
+    const unsigned half = 0xffffu << (threadIdx.x & 16);          // its lanes of the warp
+    const int64_t stride = (int64_t)gridDim.x * (blockDim.x >> 4);
     float dom = 0.0f;
 #pragma unroll
     for (int a = 0; a < 3; a++) dom = fmaxf(dom, fmaxf(fabsf(G.flo[a]), fabsf(G.fhi[a])));
-    for (int64_t q = (int64_t)blockIdx.x * (blockDim.x >> 5) + wib; q < ncand; q += nwarps) {
-        const int64_t r = order[q];
+    for (int64_t q = (int64_t)blockIdx.x * (blockDim.x >> 4) + slot; q < ncand; q += stride) {
+        // everything up to the cuts is uniform over the half warp
+        const int64_t r = order ? order[q] : q;
+        const float rwork = work[r];
+        if (!(rwork > thr)) continue;
         const Start R = starts[r];
-        const float rwork = start_work(R, work, r);
-        if (R.cur < 0 || !(rwork > thr)) continue;  // uniform over the warp
+        if (R.cur < 0) continue;
         const int K = (int)fminf((float)kMaxSegs, ceilf(rwork / W));
-        const float of[3] = {(float)o[3 * r], (float)o[3 * r + 1], (float)o[3 * r + 2]};
-        const float kf[3] = {(float)d[3 * r], (float)d[3 * r + 1], (float)d[3 * r + 2]};
+        const float of[3] = {near_float(o[3 * r]), near_float(o[3 * r + 1]), near_float(o[3 * r + 2])};
+        const float kf[3] = {near_float(d[3 * r]), near_float(d[3 * r + 1]), near_float(d[3 * r + 2])};
         const uint32_t sg = R.sg & 0x3fu;
-        // the walked interval as the setup's march took it: entry time to the domain exit or s_max
-        const float ts = (float)kdouble(R.ktstart);
-        const float tend = start_t1(R, t1, r);
+        // the walked interval as the setup's estimate took it: entry time to the domain exit or s_max
+        const float ts = near_float(kdouble(R.ktstart));
+        const float tend = t1[r];
         // cuts stay clear of both ends of the path
         const float lo_t = ts + (tend - ts) * 0x1p-10f, hi_t = tend - (tend - ts) * 0x1p-10f;
         // cut time of this lane: where the estimated work reaches (lane + 1) / K of the total.  The
-        // estimate comes from 32 samples of the work lattice, lane i at the middle of the i-th of 32
-        // equal pieces of the walked interval; a warp prefix sum gives the work up to each piece's
-        // end, and a search over it the piece where the target falls (linear inside the piece).
-        // Coarser than a cell-by-cell march, which cost each warp ~1000 instructions per long path;
-        // the cuts only balance work.
+        // estimate comes from 32 samples of the work lattice, this lane's two at the middles of pieces 2 lane
+        // and 2 lane + 1 of 32 equal pieces of the walked interval; a prefix sum gives the work up to each
+        // lane's end, and a search over it the piece where the target falls (linear inside the piece).
         const float dt = (tend - ts) * (1.0f / 32.0f);
-        float rate = 0.0f;
-        {
+        float rate[2];
+#pragma unroll
+        for (int h = 0; h < 2; h++) {
             const int N = G.work_n;
-            const float tm = ts + ((float)lane + 0.5f) * dt;
+            const float tm = ts + ((float)(2 * lane + h) + 0.5f) * dt;
             int ci[3];
 #pragma unroll
             for (int a = 0; a < 3; a++) {
                 const float lo = G.flo[a];
-                const float p = (of[a] + kf[a] * tm - lo) * ((float)N / (G.fhi[a] - lo));
+                const float p = (of[a] + kf[a] * tm - lo) * __fdividef((float)N, G.fhi[a] - lo);
                 const int c = (int)floorf(p);
                 ci[a] = c < 0 ? 0 : (c > N - 1 ? N - 1 : c);
             }
-            rate = lat[ci[0] + N * (ci[1] + N * ci[2])];
+            rate[h] = lat[ci[0] + N * (ci[1] + N * ci[2])];
         }
-        float e = rate * dt;  // inclusive prefix sum over the pieces
+        float e = (rate[0] + rate[1]) * dt;  // inclusive prefix sum over the lanes
 #pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const float v = __shfl_up_sync(0xffffffffu, e, off);
+        for (int off = 1; off < 16; off <<= 1) {
+            const float v = __shfl_up_sync(half, e, off, 16);
             if (lane >= off) e += v;
         }
-        const float E = __shfl_sync(0xffffffffu, e, 31);
+        const float E = __shfl_sync(half, e, 15, 16);
         const float target = E * (float)(lane + 1) / (float)K;
-        int pos = 0;  // first piece whose prefix reaches the target
+        int pos = 0;  // first lane whose prefix reaches the target
 #pragma unroll
-        for (int step = 16; step >= 1; step >>= 1) {
-            const float v = __shfl_sync(0xffffffffu, e, pos + step - 1);
+        for (int step = 8; step >= 1; step >>= 1) {
+            const float v = __shfl_sync(half, e, pos + step - 1, 16);
             if (v < target) pos += step;
         }
-        const float e_before = __shfl_sync(0xffffffffu, e, pos > 0 ? pos - 1 : 0);
-        const float r_pos = __shfl_sync(0xffffffffu, rate, pos);
+        const float e_prev = __shfl_sync(half, e, pos > 0 ? pos - 1 : 0, 16);
+        const float r_a = __shfl_sync(half, rate[0], pos, 16), r_b = __shfl_sync(half, rate[1], pos, 16);
+        float into = target - (pos > 0 ? e_prev : 0.0f);  // work to go from the start of that lane's first piece
+        const bool second = into > r_a * dt;
+        if (second) into -= r_a * dt;
+        const float r_pos = second ? r_b : r_a;
         const bool found = E > 0.0f && r_pos > 0.0f;
-        const float tc = found ? ts + (float)pos * dt + (target - (pos > 0 ? e_before : 0.0f)) / r_pos : 0.0f;
+        const float tc = found ? ts + (float)(2 * pos + (second ? 1 : 0)) * dt + into / r_pos : 0.0f;
         // the leaf containing o + d t_c, and whether the point lies deep inside it
         bool ok = false;
         int32_t Lid = -1;
@@ -265,39 +271,36 @@ __global__ void __launch_bounds__(256) split_kernel(const DevGrid G, int64_t n, 
                 }
             }
         }
-        // accept cuts in path order: increasing t_c, a leaf different from the previous cut's
-        int ncut = 0;
-        float tprev = ts;
-        int32_t prev_leaf = R.cur;
-        for (int j = 0; j < K - 1; j++) {
-            const bool okj = __shfl_sync(0xffffffffu, ok, j);
-            const float tj = __shfl_sync(0xffffffffu, tc, j);
-            const int32_t Lj = __shfl_sync(0xffffffffu, Lid, j);
-            if (okj && tj > tprev && Lj != prev_leaf) {
-                if (lane == j) {
-                    s_leaf[wib][ncut] = Lid;
-                    s_key[wib][ncut] = f32_key(tc);
-                }
-                ncut++;
-                tprev = tj;
-                prev_leaf = Lj;
-            }
-        }
-        __syncwarp();
+        __syncwarp(half);
+        // accept cuts in path order: later than the cut before and in another leaf (the leaves a path crosses
+        // do not recur, so that comparing with the cut before, accepted or not, is enough)
+        const unsigned oks = (__ballot_sync(half, ok) & half) >> (threadIdx.x & 16);
+        const int before = 31 - __clz(oks & ((1u << lane) - 1u));  // -1: none
+        const float t_prev = __shfl_sync(half, tc, before < 0 ? 0 : before, 16);
+        const int32_t l_prev = __shfl_sync(half, Lid, before < 0 ? 0 : before, 16);
+        const bool take = ok && tc > (before < 0 ? ts : t_prev) && Lid != (before < 0 ? R.cur : l_prev);
+        const unsigned cuts = (__ballot_sync(half, take) & half) >> (threadIdx.x & 16);
+        const int ncut = __popc(cuts);
         if (ncut == 0) continue;
+        if (take) {
+            const int c = __popc(cuts & ((1u << lane) - 1u));
+            s_leaf[slot][c] = Lid;
+            s_key[slot][c] = f32_key(tc);
+        }
+        __syncwarp(half);
         const int nseg = ncut + 1;
         unsigned long long first = 0;
         if (lane == 0) first = atomicAdd(seg_count, (unsigned long long)nseg);
-        first = __shfl_sync(0xffffffffu, first, 0);
+        first = __shfl_sync(half, first, 0, 16);
         if (first + (unsigned long long)nseg > (unsigned long long)seg_cap) {
-            for (unsigned long long s = first + lane; s < (unsigned long long)seg_cap; s += 32) {
-                SegStart E;
-                E.ktstart = 0;
-                E.ktstop = KEY_INF;
-                E.ray = r;
-                E.cur = -1;
-                E.sg = 0;
-                segs[s] = E;
+            for (unsigned long long s = first + lane; s < (unsigned long long)seg_cap; s += 16) {
+                SegStart E0;
+                E0.ktstart = 0;
+                E0.ktstop = KEY_INF;
+                E0.ray = r;
+                E0.cur = -1;
+                E0.sg = 0;
+                segs[s] = E0;
                 if constexpr (F) {
                     starts[n + (int64_t)s].cur = -1;
                     starts[n + (int64_t)s].sg = 0;
@@ -306,18 +309,18 @@ __global__ void __launch_bounds__(256) split_kernel(const DevGrid G, int64_t n, 
             continue;
         }
         if (lane < nseg) {
-            SegStart E;
-            E.ktstart = lane == 0 ? R.ktstart : s_key[wib][lane - 1];
-            E.ktstop = lane < ncut ? s_key[wib][lane] : KEY_INF;
-            E.ray = r;
-            E.cur = lane == 0 ? R.cur : s_leaf[wib][lane - 1];
-            E.sg = sg | (lane == 0 ? 0u : SG_SKIP_FIRST);
-            segs[first + lane] = E;
+            SegStart E0;
+            E0.ktstart = lane == 0 ? R.ktstart : s_key[slot][lane - 1];
+            E0.ktstop = lane < ncut ? s_key[slot][lane] : KEY_INF;
+            E0.ray = r;
+            E0.cur = lane == 0 ? R.cur : s_leaf[slot][lane - 1];
+            E0.sg = sg | (lane == 0 ? 0u : SG_SKIP_FIRST);
+            segs[first + lane] = E0;
             if constexpr (F) {  // the segment's start record
                 RayStartF B = R;
-                B.ktstart = E.ktstart;
-                B.cur = E.cur;
-                B.sg = E.sg | (R.sg & SG_EXACT);
+                B.ktstart = E0.ktstart;
+                B.cur = E0.cur;
+                B.sg = E0.sg | (R.sg & SG_EXACT);
                 starts[n + (int64_t)first + lane] = B;
             }
         }
@@ -330,7 +333,7 @@ __global__ void __launch_bounds__(256) split_kernel(const DevGrid G, int64_t n, 
             list[i] = rec;
             starts[r].sg = R.sg | SG_SPLIT;
         }
-        __syncwarp();
+        __syncwarp(half);
     }
 }
 
@@ -663,6 +666,7 @@ hg_status make_plan(hg_rays &P, const hg_grid *g, int64_t n, const double *o, co
     P.threads = blocks * block;
     // auto schedule: order by estimated work only when each resident thread
     // gets few paths (then the heaviest paths would otherwise set the end)
+    const bool automatic = schedule == 0;
     if (schedule == 0) schedule = (n < 48 * P.threads) ? 3 : 2;
     P.dyn = (schedule >= 2);
     P.ordered = (schedule == 3);
@@ -672,6 +676,9 @@ hg_status make_plan(hg_rays &P, const hg_grid *g, int64_t n, const double *o, co
         if (hs != HG_OK) return hs;
         P.threads = blocks * block;
     }
+    // with a thread for every ray the order of the queue does not matter: no sorting pass unless the caller
+    // chose the schedule or the splitting
+    if (automatic && P.splitting && split == HG_SPLIT_AUTO && n <= P.threads) P.ordered = false;
     P.seg_cap = P.splitting ? std::min<int64_t>((split == HG_SPLIT_FORCE ? 16 * n : 3 * P.threads) + 1024, 16 * n)
                             : 0;
     // scratch: start records; the queue counter; for the ordered schedule the
@@ -681,9 +688,10 @@ hg_status make_plan(hg_rays &P, const hg_grid *g, int64_t n, const double *o, co
     auto al = [](size_t b) { return (b + 255) / 256 * 256; };
     // (single-precision grids: start records of the segments after those of the rays)
     const size_t start_bytes = al(f32 ? (size_t)(n + P.seg_cap) * sizeof(RayStartF) : (size_t)n * sizeof(RayStart));
-    const size_t t1_bytes = P.splitting && f32 ? al((size_t)n * sizeof(float)) : 0;
+    const size_t t1_bytes = P.splitting ? al((size_t)n * sizeof(float)) : 0;
     const size_t order_bytes = P.ordered ? al((size_t)n * sizeof(int64_t)) : 0;
-    const size_t work_bytes = P.ordered ? al((size_t)n * sizeof(float)) : 0;
+    const bool estimate = (P.ordered || P.splitting) && !exact && g->d.work;
+    const size_t work_bytes = P.ordered || P.splitting ? al((size_t)n * sizeof(float)) : 0;
     const size_t count_bytes = al((2 * kBuckets + 4) * sizeof(unsigned long long));
     const size_t seg_bytes = al((size_t)P.seg_cap * sizeof(SegStart));
     const size_t acc_bytes = al((size_t)P.seg_cap * sizeof(double));
@@ -726,9 +734,9 @@ hg_status make_plan(hg_rays &P, const hg_grid *g, int64_t n, const double *o, co
     const int64_t sblocks = std::min<int64_t>((n + 255) / 256, (int64_t)sm_count() * 8);
     const int snodes = setup_nodes(g);
     const size_t setup_smem = geo_offset((size_t)snodes * node_bytes_of(g->d)) +
-                              ((P.ordered && !exact && g->d.work) ? kLatticeBytes : 0);
+                              (estimate ? kLatticeBytes : 0);
     pick_setup(g->d.kind, f32)<<<(unsigned)sblocks, 256, setup_smem, stream>>>(
-        g->d, n, o, d, smax, P.starts, snodes, P.counts, exact, P.ordered ? P.work_total : nullptr, P.work, P.t1);
+        g->d, n, o, d, smax, P.starts, snodes, P.counts, exact, P.splitting ? P.work_total : nullptr, P.work, P.t1);
     note_launches(1);
     if (P.ordered) {
         order_kernel<<<(unsigned)sblocks, 256, 0, stream>>>(n, P.work, P.counts, P.counts + kBuckets, P.order);
@@ -736,14 +744,14 @@ hg_status make_plan(hg_rays &P, const hg_grid *g, int64_t n, const double *o, co
     }
     if (P.splitting) {
         const int force = split == HG_SPLIT_FORCE ? 1 : 0;
-        // one warp per candidate ray: as many blocks as are resident at once
+        // half a warp per candidate ray: as many blocks as are resident at once
         const unsigned pblocks = (unsigned)sm_count() * 4;
         const auto split_fn = f32 ? (g->d.kind == HG_KDTREE ? &split_kernel<HG_KDTREE, true>
                                                             : &split_kernel<HG_OCTREE, true>)
                                   : (g->d.kind == HG_KDTREE ? &split_kernel<HG_KDTREE, false>
                                                             : &split_kernel<HG_OCTREE, false>);
-        split_fn<<<pblocks, 256, 0, stream>>>(g->d, n, o, d, smax, P.starts, P.work, P.t1, P.work_total, P.counts,
-                                              P.order, P.threads, force, P.segs, P.seg_cap, P.seg_count, P.list,
+        split_fn<<<pblocks, 256, 0, stream>>>(g->d, n, o, d, P.starts, P.work, P.t1, P.work_total, P.counts, P.order,
+                                              P.threads, force, P.segs, P.seg_cap, P.seg_count, P.list,
                                               P.split_count);
         note_launches(1);
     }

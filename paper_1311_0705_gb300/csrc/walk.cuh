@@ -242,59 +242,35 @@ __device__ __forceinline__ void stage_lattice(const DevGrid &G, float *lat) {
     for (int i = threadIdx.x; i < kWorkN * kWorkN * kWorkN / 4; i += blockDim.x) dst[i] = __ldg(src + i);
 }
 
-// March of the path o + t k, t in [t0, t1], through the coarse work
-// lattice (expected crossings per unit length, G.work, or its copy in
-// shared memory lat): a 3-D DDA (Amanatides & Woo, 1987) in single
-// precision.  Calls f(t, tn, rate, e)
-// for every lattice cell the path crosses, [t, tn] being the part inside
-// it and e the work before it; returns the total work.  It only orders and
-// cuts the work; it never affects a result.
-template <class F>
-__device__ __forceinline__ float work_march(const DevGrid &G, const float *lat, const float *o, const float *k,
-                                            float t0, float t1, F &&f) {
-    const int N = G.work_n;
-    if (!G.work || N <= 0 || !(t1 > t0)) return 0.0f;
-    float tmax[3], tdel[3];
-    int c[3], step[3];
+// Estimated crossings of the path o + t k, t in [t0, t1]: the coarse work lattice (expected crossings per
+// unit length, G.work or its copy lat in shared memory) sampled at the middle of kWorkSamples equal pieces.
+// It only orders and cuts the work; it never affects a result.  A cell-by-cell march of the path (3-D DDA)
+// ended after another number of cells on every lane, up to 48, and took most of the setup pass's
+// instructions: 1e6 rays on the disk octree 187 us, with the samples (and 1/d by the reciprocal function) 102 us.
+constexpr int kWorkSamples = 16;
+__device__ __forceinline__ float work_estimate(const DevGrid &G, const float *lat, const float *o, const float *k,
+                                               float t0, float t1) {
+    static_assert(kWorkN == 16, "cells are taken from the low four bits");
+    if (!(t1 > t0)) return 0.0f;
+    // cell number = floor of the lattice coordinate, read off the low mantissa bits of (coordinate - 1/2) + 2^23
+    // rounded to a whole number (a coordinate on a cell's edge may count for either side)
+    const float dt = (t1 - t0) * (1.0f / (float)kWorkSamples);
+    float p[3], dp[3];
 #pragma unroll
     for (int a = 0; a < 3; a++) {
-        const float lo = G.flo[a];
-        const float sc = (float)N / (G.fhi[a] - lo);
-        const float ka = k[a] * sc;  // lattice units per unit t
-        const float p = (o[a] + k[a] * t0 - lo) * sc;
-        int ci = (int)floorf(p);
-        ci = ci < 0 ? 0 : (ci > N - 1 ? N - 1 : ci);
-        c[a] = ci;
-        if (ka > 0.0f) {
-            tdel[a] = 1.0f / ka;
-            tmax[a] = t0 + ((float)(ci + 1) - p) * tdel[a];
-            step[a] = 1;
-        } else if (ka < 0.0f) {
-            tdel[a] = -1.0f / ka;
-            tmax[a] = t0 + (p - (float)ci) * tdel[a];
-            step[a] = -1;
-        } else {
-            tdel[a] = 0.0f;
-            tmax[a] = CUDART_INF_F;
-            step[a] = 0;
-        }
+        const float sc = __fdividef((float)kWorkN, G.fhi[a] - G.flo[a]);
+        dp[a] = k[a] * dt * sc;
+        p[a] = (o[a] + k[a] * t0 - G.flo[a]) * sc - 0.5f + 0.5f * dp[a];
     }
-    float t = t0;
     float e = 0.0f;
-    for (int it = 0; it < 3 * N + 3; it++) {
-        const int ax = (tmax[0] <= tmax[1]) ? (tmax[0] <= tmax[2] ? 0 : 2) : (tmax[1] <= tmax[2] ? 1 : 2);
-        float tn = fminf(tmax[ax], t1);
-        if (tn < t) tn = t;
-        const float rate = lat[c[0] + N * (c[1] + N * c[2])];
-        f(t, tn, rate, e);
-        e += rate * (tn - t);
-        t = tn;
-        if (!(tmax[ax] < t1)) break;
-        c[ax] += step[ax];
-        if (c[ax] < 0 || c[ax] >= N) break;
-        tmax[ax] += tdel[ax];
+#pragma unroll
+    for (int j = 0; j < kWorkSamples; j++) {
+        const uint32_t x = __float_as_uint(__fmaf_rn((float)j, dp[0], p[0]) + 0x1p23f) & 15u;
+        const uint32_t y = __float_as_uint(__fmaf_rn((float)j, dp[1], p[1]) + 0x1p23f) & 15u;
+        const uint32_t z = __float_as_uint(__fmaf_rn((float)j, dp[2], p[2]) + 0x1p23f) & 15u;
+        e += lat[x | y << 4 | z << 8];
     }
-    return e;
+    return e * dt;
 }
 
 // Nearest single-precision value of a double (half away from zero; below 2^-126: zero), by integer
@@ -324,7 +300,7 @@ __device__ __forceinline__ bool dlt0(double x) { return __double_as_longlong(x) 
 template <class Locate>
 __device__ __forceinline__ RayStart ray_setup(const DevGrid &G, Locate &&locate, const double *__restrict__ o,
                                               const double *__restrict__ d, const double *__restrict__ smax,
-                                              int64_t r, bool estimate = false, const float *lat = nullptr) {
+                                              int64_t r, const float *lat = nullptr) {
     RayStart R;
     R.ik0 = R.ik1 = R.ik2 = 0.0;
     R.ktstart = 0;
@@ -352,7 +328,7 @@ __device__ __forceinline__ RayStart ray_setup(const DevGrid &G, Locate &&locate,
     bool inside = true;
 #pragma unroll
     for (int a = 0; a < 3; a++) {
-        ik[a] = dzero(kk[a]) ? 0.0 : 1.0 / kk[a];
+        ik[a] = dzero(kk[a]) ? 0.0 : __drcp_rn(kk[a]);
         sg |= (dgt0(kk[a]) ? 1u : 0u) << a;
         sg |= (dlt0(kk[a]) ? 1u : 0u) << (3 + a);
         ko[a] = okey(oo[a]);
@@ -420,10 +396,10 @@ __device__ __forceinline__ RayStart ray_setup(const DevGrid &G, Locate &&locate,
     R.cur = c;
     R.sg = sg;
     R.t1 = t1f;
-    if (estimate) {
+    if (lat) {
         const float of[3] = {near_float(oo[0]), near_float(oo[1]), near_float(oo[2])};
         const float kf[3] = {near_float(kk[0]), near_float(kk[1]), near_float(kk[2])};
-        R.work = work_march(G, lat ? lat : G.work, of, kf, near_float(ts), t1f, [](float, float, float, float) {});
+        R.work = work_estimate(G, lat, of, kf, near_float(ts), t1f);
     }
     return R;
 }
