@@ -546,7 +546,7 @@ __global__ void __launch_bounds__(32 * kTauWarps, 2) disk_tau_kernel(const DevMo
 // Deterministic two-pass statistics in three launches: per-block sums of x = a - b; per-block sums of
 // (x - mean)^2, every block adding up the first pass's sums for itself; one block for the results.
 // 1e6 values: 40 us with a launch of one block after each pass and one chain of additions per thread, now
-// DIFF_US us (the two passes read 32 MB, mostly from L2, and are over in a few FP64 latencies of 76 cycles).
+// 27 (see the FP64 instructions: a serial sum of 8 by every thread of 977 blocks alone took 4 us).
 constexpr int kStatBlock = 256;
 __device__ __forceinline__ double block_sum(double v, double *sh) {
     for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);

@@ -125,15 +125,18 @@ struct SplitRec {
 // max(64, A), A = total / T the mean work per thread of the walking launch
 // (only those can outlast the launch's bulk when the heaviest go first),
 // into K = min(16, ceil(w / W)) pieces of equal estimated work,
-// W = max(32, A / 2).  Forced: every ray of more than 3 estimated crossings,
-// W = 2.  Half a warp per ray (a ray has at most 15 cuts), over the heavy
+// W = max(32, A / 2).  Without a sorted queue (a thread for every ray) the launch lasts
+// as long as its longest item: max(18, 3 A / 4) and W = max(12, A / 2).  (1e4 rays with
+// emission: 167 -> 128 us; on sorted batches of 2e5 and 3e5 rays the additional paths
+// cost the planner more than the walk gained, 219 -> 253 and 706 -> 784 us.)
+// Forced: every ray of more than 3 estimated crossings, W = 2.  Half a warp per ray (a ray has at most 15 cuts), over the heavy
 // end of the work-ordered queue, or over all rays when there is none: the
 // lanes sample the work lattice at 32 points of the path and sum them
 // (a prefix sum), lane j places cut j where the sum reaches (j + 1) / K
 // of the total (descent and depth test), and the accepted cuts are those of
 // increasing t_c in distinct leaves, in path order.  Segment slots are
 // taken with one atomic per ray; their count is bounded (sum over split
-// rays of ceil(w/W) <= total/W + total/max(64, A) <= 3 T, or 16 n when
+// rays of ceil(w/W) <= total/W + total/threshold <= 3.4 T, or 16 n when
 // forced), so seg_cap is never reached -- if it were, the ray would stay
 // whole and the slots taken would be marked empty.
 // A ray's chain of dependent loads (queue, start record, one per tree level,
@@ -159,8 +162,8 @@ __global__ void __launch_bounds__(256) split_kernel(const DevGrid G, int64_t n, 
     if (!G.work || G.work_n <= 0) return;
     stage_lattice(G, lat);
     const float A = (float)*work_total / (float)threads;
-    const float W = force ? 2.0f : fmaxf(32.0f, 0.5f * A);
-    const float thr = force ? 3.0f : fmaxf(64.0f, A);
+    const float W = force ? 2.0f : fmaxf(order ? 32.0f : 12.0f, 0.5f * A);
+    const float thr = force ? 3.0f : (order ? fmaxf(64.0f, A) : fmaxf(18.0f, 0.75f * A));
     if (threadIdx.x == 0) {
         // the queue is sorted by work bucket: candidates are the buckets up to that of the threshold
         long long c = n;
@@ -343,7 +346,9 @@ __global__ void __launch_bounds__(256) split_kernel(const DevGrid G, int64_t n, 
 __global__ void __launch_bounds__(256) seg_base_kernel(const SplitRec *__restrict__ list,
                                                        const unsigned long long *split_count,
                                                        const int64_t *__restrict__ seg_off,
-                                                       const int32_t *__restrict__ part_nc, int64_t *seg_base) {
+                                                       const int32_t *__restrict__ part_nc, int64_t *seg_base,
+                                                       const uint32_t *run_if) {
+    if (run_if && *run_if == 0u) return;
     const int64_t m = (int64_t)*split_count;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
         const SplitRec rec = list[i];
@@ -364,7 +369,8 @@ __global__ void __launch_bounds__(256) combine_kernel(const SplitRec *__restrict
                                                       const int32_t *__restrict__ part_nc,
                                                       const int32_t *__restrict__ part_last,
                                                       const uint8_t *__restrict__ part_st, double kappa, void *tau,
-                                                      int32_t *ncross, uint8_t *status) {
+                                                      int32_t *ncross, uint8_t *status, const uint32_t *run_if) {
+    if (run_if && *run_if == 0u) return;
     const int64_t m = (int64_t)*split_count;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
         const SplitRec rec = list[i];
@@ -679,7 +685,7 @@ hg_status make_plan(hg_rays &P, const hg_grid *g, int64_t n, const double *o, co
     // with a thread for every ray the order of the queue does not matter: no sorting pass unless the caller
     // chose the schedule or the splitting
     if (automatic && P.splitting && split == HG_SPLIT_AUTO && n <= P.threads) P.ordered = false;
-    P.seg_cap = P.splitting ? std::min<int64_t>((split == HG_SPLIT_FORCE ? 16 * n : 3 * P.threads) + 1024, 16 * n)
+    P.seg_cap = P.splitting ? std::min<int64_t>((split == HG_SPLIT_FORCE ? 16 * n : 4 * P.threads) + 1024, 16 * n)
                             : 0;
     // scratch: start records; the queue counter; for the ordered schedule the
     // queue, work estimates and counters (bucket counts and fills, work
@@ -745,7 +751,7 @@ hg_status make_plan(hg_rays &P, const hg_grid *g, int64_t n, const double *o, co
     if (P.splitting) {
         const int force = split == HG_SPLIT_FORCE ? 1 : 0;
         // half a warp per candidate ray: as many blocks as are resident at once
-        const unsigned pblocks = (unsigned)sm_count() * 4;
+        const unsigned pblocks = (unsigned)std::min<int64_t>((int64_t)sm_count() * 4, (n + kPlanRays - 1) / kPlanRays);
         const auto split_fn = f32 ? (g->d.kind == HG_KDTREE ? &split_kernel<HG_KDTREE, true>
                                                             : &split_kernel<HG_OCTREE, true>)
                                   : (g->d.kind == HG_KDTREE ? &split_kernel<HG_KDTREE, false>
@@ -1066,7 +1072,8 @@ hg_status walk_plan(hg_rays &P, int mode, int prec, TraceArgs A, cudaStream_t st
     const unsigned cblocks =
         (unsigned)std::max<int64_t>(1, std::min<int64_t>((P.seg_cap / 2 + 255) / 256, (int64_t)sm_count() * 4));
     if (P.splitting && mode == MODE_FILL) {
-        seg_base_kernel<<<cblocks, 256, 0, stream>>>(P.list, P.split_count, A.seg_off, P.part_nc, P.seg_base);
+        seg_base_kernel<<<cblocks, 256, 0, stream>>>(P.list, P.split_count, A.seg_off, P.part_nc, P.seg_base,
+                                                     A.run_if);
         note_launches(1);
     }
     k<<<(unsigned)blocks, P.block, P.walk_smem, stream>>>(A);
@@ -1077,19 +1084,19 @@ hg_status walk_plan(hg_rays &P, int mode, int prec, TraceArgs A, cudaStream_t st
             if ((prec & 1) == HG_FP64)
                 combine_kernel<MODE_TAU, HG_FP64><<<cblocks, 256, 0, stream>>>(
                     P.list, P.split_count, P.segs, P.part_acc, P.part_nc, P.part_last, P.part_st, A.kappa, A.tau,
-                    A.ncross, A.status);
+                    A.ncross, A.status, A.run_if);
             else
                 combine_kernel<MODE_TAU, HG_FP32K><<<cblocks, 256, 0, stream>>>(
                     P.list, P.split_count, P.segs, P.part_acc, P.part_nc, P.part_last, P.part_st, A.kappa, A.tau,
-                    A.ncross, A.status);
+                    A.ncross, A.status, A.run_if);
         } else if (mode == MODE_FILL) {
             combine_kernel<MODE_FILL, 0><<<cblocks, 256, 0, stream>>>(P.list, P.split_count, P.segs, P.part_acc,
                                                                     P.part_nc, P.part_last, P.part_st, A.kappa,
-                                                                    nullptr, nullptr, A.status);
+                                                                    nullptr, nullptr, A.status, A.run_if);
         } else {
             combine_kernel<MODE_ADJ, 0><<<cblocks, 256, 0, stream>>>(P.list, P.split_count, P.segs, P.part_acc,
                                                                    P.part_nc, P.part_last, P.part_st, A.kappa,
-                                                                   nullptr, nullptr, A.status);
+                                                                   nullptr, nullptr, A.status, A.run_if);
         }
         note_launches(1);
         e = cudaGetLastError();
