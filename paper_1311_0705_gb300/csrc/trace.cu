@@ -151,7 +151,7 @@ __global__ void __launch_bounds__(256) split_kernel(const DevGrid G, int64_t n, 
                                                     const unsigned long long *work_total,
                                                     const unsigned long long *bucket_count,
                                                     const int64_t *__restrict__ order, int64_t threads, int force,
-                                                    SegStart *segs, int64_t seg_cap, unsigned long long *seg_count,
+                                                    int n_smem, SegStart *segs, int64_t seg_cap, unsigned long long *seg_count,
                                                     SplitRec *list, unsigned long long *split_count) {
     using Start = typename std::conditional<F, RayStartF, RayStart>::type;
     Start *starts = static_cast<Start *>(starts_v);
@@ -159,6 +159,7 @@ __global__ void __launch_bounds__(256) split_kernel(const DevGrid G, int64_t n, 
     __shared__ long long s_key[kPlanRays][kMaxSegs];
     __shared__ long long s_ncand;
     __shared__ __align__(16) float lat[kWorkN * kWorkN * kWorkN];
+    extern __shared__ __align__(16) unsigned char snodes[];  // the top n_smem nodes, where the descents start
     if (!G.work || G.work_n <= 0) return;
     stage_lattice(G, lat);
     const float A = (float)*work_total / (float)threads;
@@ -174,7 +175,7 @@ __global__ void __launch_bounds__(256) split_kernel(const DevGrid G, int64_t n, 
         }
         s_ncand = c;
     }
-    __syncthreads();
+    stage_nodes(G.nodes, n_smem * node_size<KIND, F>(), snodes);
     const long long ncand = s_ncand;
     const int lane = threadIdx.x & 15, slot = threadIdx.x >> 4;  // lane of the half warp, ray slot in the block
     const unsigned half = 0xffffu << (threadIdx.x & 16);          // its lanes of the warp
@@ -239,38 +240,54 @@ __global__ void __launch_bounds__(256) split_kernel(const DevGrid G, int64_t n, 
         if (second) into -= r_a * dt;
         const float r_pos = second ? r_b : r_a;
         const bool found = E > 0.0f && r_pos > 0.0f;
-        const float tc = found ? ts + (float)(2 * pos + (second ? 1 : 0)) * dt + into / r_pos : 0.0f;
-        // the leaf containing o + d t_c, and whether the point lies deep inside it
+        float tc = found ? ts + (float)(2 * pos + (second ? 1 : 0)) * dt + into / r_pos : 0.0f;
+        // the leaf containing o + d t_c; the cut moves to the middle of the path's way through it (a cut left where
+        // the work adds up was too near a face for the test below in one case of ten, and pieces grew
+        // to four times their size)
         bool ok = false;
         int32_t Lid = -1;
         if (lane < K - 1 && found && tc > lo_t && tc < hi_t) {
-            long long q3[3];
-            float xm[3], xp[3];
-#pragma unroll
-            for (int a = 0; a < 3; a++) {
-                const float x = of[a] + kf[a] * tc;
-                const float m = (fabsf(of[a]) + fabsf(kf[a] * tc) + dom) * 0x1p-18f;
-                q3[a] = f32_key(x);
-                xm[a] = x - m;
-                xp[a] = x + m;
-            }
-            if (in_axis(q3[0], G.klo[0], G.khi[0], dpos(sg, 0), dneg(sg, 0), true) &&
-                in_axis(q3[1], G.klo[1], G.khi[1], dpos(sg, 1), dneg(sg, 1), true) &&
-                in_axis(q3[2], G.klo[2], G.khi[2], dpos(sg, 2), dneg(sg, 2), true))
-                Lid = F ? locate_key_f<KIND>(G, nullptr, 0, q3[0], q3[1], q3[2], sg)
-                        : descend<KIND>(G, nullptr, 0, q3[0], q3[1], q3[2], sg);
+            const long long q0 = f32_key(of[0] + kf[0] * tc), q1 = f32_key(of[1] + kf[1] * tc),
+                            q2 = f32_key(of[2] + kf[2] * tc);
+            if (in_axis(q0, G.klo[0], G.khi[0], dpos(sg, 0), dneg(sg, 0), true) &&
+                in_axis(q1, G.klo[1], G.khi[1], dpos(sg, 1), dneg(sg, 1), true) &&
+                in_axis(q2, G.klo[2], G.khi[2], dpos(sg, 2), dneg(sg, 2), true))
+                Lid = F ? locate_key_f<KIND>(G, snodes, n_smem, q0, q1, q2, sg)
+                        : descend<KIND>(G, snodes, n_smem, q0, q1, q2, sg);
             if (Lid >= 0) {
-                ok = true;
+                float lo[3], hi[3];
                 if (F) {
-                    const LeafRecF *L = G.recf + Lid;
 #pragma unroll
-                    for (int a = 0; a < 3; a++) ok = ok && xm[a] >= __ldg(&L->lo[a]) && xp[a] <= __ldg(&L->hi[a]);
+                    for (int a = 0; a < 3; a++) {
+                        lo[a] = __ldg(&G.recf[Lid].lo[a]);
+                        hi[a] = __ldg(&G.recf[Lid].hi[a]);
+                    }
                 } else {
                     Leaf L;
                     load_leaf(G.rec, Lid, L);
 #pragma unroll
-                    for (int a = 0; a < 3; a++)
-                        ok = ok && f32_key(xm[a]) >= L.lo(a) && f32_key(xp[a]) <= L.hi(a);
+                    for (int a = 0; a < 3; a++) {
+                        lo[a] = near_float(kdouble(L.lo(a)));
+                        hi[a] = near_float(kdouble(L.hi(a)));
+                    }
+                }
+                float t_in = lo_t, t_out = hi_t;
+#pragma unroll
+                for (int a = 0; a < 3; a++) {
+                    const float t_lo = __fdividef(lo[a] - of[a], kf[a]), t_hi = __fdividef(hi[a] - of[a], kf[a]);
+                    if (kf[a] != 0.0f) {
+                        t_in = fmaxf(t_in, fminf(t_lo, t_hi));
+                        t_out = fminf(t_out, fmaxf(t_lo, t_hi));
+                    }
+                }
+                tc = 0.5f * (t_in + t_out);
+                // deep inside: by the margin below and by what rounding wide bounds to single precision can add
+                ok = tc > lo_t && tc < hi_t;
+#pragma unroll
+                for (int a = 0; a < 3; a++) {
+                    const float x = of[a] + kf[a] * tc;
+                    const float m = (fabsf(of[a]) + fabsf(kf[a] * tc) + dom) * 0x1p-18f;
+                    ok = ok && x - m >= lo[a] && x + m <= hi[a];
                 }
             }
         }
@@ -756,9 +773,10 @@ hg_status make_plan(hg_rays &P, const hg_grid *g, int64_t n, const double *o, co
                                                             : &split_kernel<HG_OCTREE, true>)
                                   : (g->d.kind == HG_KDTREE ? &split_kernel<HG_KDTREE, false>
                                                             : &split_kernel<HG_OCTREE, false>);
-        split_fn<<<pblocks, 256, 0, stream>>>(g->d, n, o, d, P.starts, P.work, P.t1, P.work_total, P.counts, P.order,
-                                              P.threads, force, P.segs, P.seg_cap, P.seg_count, P.list,
-                                              P.split_count);
+        const size_t psmem = geo_offset((size_t)snodes * node_bytes_of(g->d));
+        split_fn<<<pblocks, 256, psmem, stream>>>(g->d, n, o, d, P.starts, P.work, P.t1, P.work_total, P.counts, P.order,
+                                                  P.threads, force, snodes, P.segs, P.seg_cap, P.seg_count, P.list,
+                                                  P.split_count);
         note_launches(1);
     }
     e = cudaGetLastError();
