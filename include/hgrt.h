@@ -13,7 +13,10 @@
  *     are returned synchronously as hg_status; a kernel fault surfaces on
  *     the caller's next synchronisation.  Scratch memory these calls need
  *     is taken from the CUDA stream-ordered allocator on the same stream
- *     and released on it before the call returns.
+ *     and released on it before the call returns; while a grid or ray plan
+ *     of the device is alive, up to 2 GiB per device of released scratch is
+ *     kept for later calls on the same stream (not under stream capture:
+ *     a graph's scratch is its own), and freed with the last of them.
  *   - Per-ray problems never abort a launch: they are reported as bit
  *     flags (HG_RAY_*) in the optional per-ray status array.
  *   - hg_last_error() returns a message for the calling thread's last

@@ -33,6 +33,7 @@ UNITS = [
     ("grid.cpp", False),
     ("build.cpp", False),
     ("common.cpp", False),
+    ("scratch.cpp", False),
 ]
 
 

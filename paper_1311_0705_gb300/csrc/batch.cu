@@ -14,6 +14,7 @@
 #include <vector>
 
 #include "hg_internal.h"
+#include "scratch.h"
 #include "trace_args.cuh"
 #include "walkf.cuh"
 
@@ -296,9 +297,10 @@ extern "C" hg_status hg_batch_trace(hg_batch *b, const double *o, const double *
     // start records of either kind, indexed by ray: two queues never share a record's bytes
     const size_t rec = b->q[1].total > 0 ? sizeof(RayStartF) : sizeof(RayStart);
     const size_t both = b->q[0].total > 0 && b->q[1].total > 0 ? (size_t)b->total * sizeof(RayStart) : 0;
-    unsigned char *starts = nullptr;
-    cudaError_t e = cudaMallocAsync((void **)&starts, (size_t)b->total * rec + both, s);
+    Scratch scratch;
+    cudaError_t e = scratch_get(scratch, (size_t)b->total * rec + both, s);
     if (e != cudaSuccess) return cuda_err(e, "batch start scratch");
+    unsigned char *starts = static_cast<unsigned char *>(scratch.p);
     for (int f = 0; f < 2 && e == cudaSuccess; f++) {
         const hg_batch::Queue &Q = b->q[f];
         if (Q.total == 0) continue;
@@ -325,7 +327,7 @@ extern "C" hg_status hg_batch_trace(hg_batch *b, const double *o, const double *
         note_launches(2);
         e = cudaGetLastError();
     }
-    cudaFreeAsync(starts, s);
+    scratch_put(scratch, s);
     return e == cudaSuccess ? HG_OK : cuda_err(e, "batch launch");
 }
 

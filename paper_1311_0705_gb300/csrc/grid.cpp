@@ -11,6 +11,7 @@
 #include <vector>
 
 #include "hg_internal.h"
+#include "scratch.h"
 
 namespace {
 
@@ -659,6 +660,8 @@ hg_status load_grid_impl(const hg_grid_desc *desc, const int32_t *ropes, int32_t
         I.device_bytes = (int64_t)(rec_bytes + tail.size() * 4 + nodes.size() +
                                    work.size() * sizeof(float));
         I.long_walls = long_walls;
+        hg::scratch_users(g->device, 1);
+        g->scratch_user = true;
         I.nav = ropes ? HG_NAV_ROPES : HG_NAV_NEIGHBOR_LISTS;
         I.reserved = 0;
         for (int a = 0; a < 3; a++) {
@@ -685,6 +688,7 @@ extern "C" void hg_free_grid(hg_grid *g) {
     if (g->d_nodes) cudaFree(g->d_nodes);
     if (g->d_work) cudaFree(g->d_work);
     if (cur != g->device) cudaSetDevice(cur);
+    if (g->scratch_user) hg::scratch_users(g->device, -1);
     delete g;
 }
 

@@ -147,6 +147,7 @@ struct hg_grid {
     void *d_nodes = nullptr;
     void *d_work = nullptr;
     int device = 0;
+    bool scratch_user = false;  // counted among the scratch's users (scratch.h)
     hg::TuneEntry tuned[2];
 };
 

@@ -8,6 +8,7 @@
 #include <vector>
 
 #include "hg_internal.h"
+#include "scratch.h"
 
 namespace hg {
 hg_status cuda_err(cudaError_t e, const char *what);
@@ -692,14 +693,15 @@ extern "C" hg_status hg_diff_stats(int64_t n, const double *a, const double *b, 
     cudaStream_t s = (cudaStream_t)stream;
     const int parts = (int)std::max<int64_t>(
         1, std::min<int64_t>((n + 4 * kStatBlock - 1) / (4 * kStatBlock), (int64_t)sm_count() * 2));
-    double *part = nullptr;
-    cudaError_t e = cudaMallocAsync((void **)&part, 2 * (size_t)parts * sizeof(double), s);
+    Scratch scratch;
+    cudaError_t e = scratch_get(scratch, 2 * (size_t)parts * sizeof(double), s);
     if (e != cudaSuccess) return cuda_err(e, "diff stats scratch");
+    double *part = static_cast<double *>(scratch.p);
     diff_partial<false><<<parts, kStatBlock, 0, s>>>(n, a, b, parts, nullptr, part);
     diff_partial<true><<<parts, kStatBlock, 0, s>>>(n, a, b, parts, part, part + parts);
     diff_final<<<1, kStatBlock, 0, s>>>(n, parts, part, part + parts, out);
     note_launches(3);
     e = cudaGetLastError();
-    cudaFreeAsync(part, s);
+    scratch_put(scratch, s);
     return e == cudaSuccess ? HG_OK : cuda_err(e, "diff stats launch");
 }

@@ -9,6 +9,7 @@
 #include <type_traits>
 
 #include "hg_internal.h"
+#include "scratch.h"
 #include "trace_args.cuh"
 #include "walkf.cuh"
 
@@ -635,7 +636,8 @@ struct hg_rays {
     bool dyn = false, ordered = false, splitting = false;
     bool traced = false;  // an optical-depth walk recorded the segments' crossing counts
     size_t walk_smem = 0;  // top tree nodes and the threads' ray geometry (the walks)
-    unsigned char *scratch = nullptr;
+    hg::Scratch scratch;
+    int device = -1;  // (prepared rays) counted among the scratch's users of this device
     void *starts = nullptr;  // RayStart, or RayStartF on a grid with single-precision records
     int64_t *order = nullptr;
     float *work = nullptr, *t1 = nullptr;
@@ -649,16 +651,14 @@ struct hg_rays {
     hg::SplitRec *list = nullptr;
     int64_t seg_cap = 0;
     // emission staging, allocated by the first staged trace
-    unsigned char *stg = nullptr;
-    size_t stg_bytes = 0;
+    hg::Scratch stg;
     void *stg_ent = nullptr;
     uint32_t *stg_next = nullptr, *stg_start_ray = nullptr, *stg_start_seg = nullptr, *stg_overflow = nullptr;
     unsigned long long *stg_ctr = nullptr;
     uint32_t stg_nchunks = 0;
     int stg_prec = -1;    // precision of the staged lengths; -1: nothing staged
     // gradient scratch: 2^k slots >= n_leaves, leaf c accumulated at slot (c * gscr_mul) & gscr_mask
-    void *gscr = nullptr;
-    size_t gscr_bytes = 0;
+    hg::Scratch gscr;
     uint32_t gscr_mul = 0, gscr_mask = 0;
 };
 
@@ -724,14 +724,11 @@ hg_status make_plan(hg_rays &P, const hg_grid *g, int64_t n, const double *o, co
     const size_t list_bytes = al((size_t)(P.seg_cap / 2) * sizeof(SplitRec));
     const size_t total_bytes = start_bytes + order_bytes + work_bytes + count_bytes + seg_bytes + acc_bytes +
                                2 * i32_bytes + u8_bytes + base_bytes + list_bytes + t1_bytes;
-    cudaError_t e = cudaMallocAsync((void **)&P.scratch, total_bytes, stream);
-    if (e != cudaSuccess) {
-        P.scratch = nullptr;
-        return cuda_err(e, "ray plan scratch");
-    }
+    cudaError_t e = scratch_get(P.scratch, total_bytes, stream);
+    if (e != cudaSuccess) return cuda_err(e, "ray plan scratch");
     size_t off = 0;
     auto take = [&](size_t b) {
-        unsigned char *q = b ? P.scratch + off : nullptr;
+        unsigned char *q = b ? static_cast<unsigned char *>(P.scratch.p) + off : nullptr;
         off += b;
         return q;
     };
@@ -784,14 +781,9 @@ hg_status make_plan(hg_rays &P, const hg_grid *g, int64_t n, const double *o, co
 }
 
 void free_plan(hg_rays &P, cudaStream_t stream) {
-    if (P.scratch) cudaFreeAsync(P.scratch, stream);
-    P.scratch = nullptr;
-    if (P.stg) cudaFreeAsync(P.stg, stream);
-    P.stg = nullptr;
-    P.stg_bytes = 0;
-    if (P.gscr) cudaFreeAsync(P.gscr, stream);
-    P.gscr = nullptr;
-    P.gscr_bytes = 0;
+    scratch_put(P.scratch, stream);
+    scratch_put(P.stg, stream);
+    scratch_put(P.gscr, stream);
 }
 
 // The gradient walks and the copy of a plan scatter into a zeroed scratch
@@ -807,22 +799,16 @@ hg_status grad_scratch_begin(hg_rays &P, int gp, TraceArgs &A, cudaStream_t stre
     int k = 0;
     while (((int64_t)1 << k) < nl) k++;
     const size_t bytes = ((size_t)1 << k) * (gp == 0 ? sizeof(double) : sizeof(float));
-    if (bytes > P.gscr_bytes) {
-        if (P.gscr) cudaFreeAsync(P.gscr, stream);
-        P.gscr = nullptr;
-        P.gscr_bytes = 0;
-        cudaError_t e = cudaMallocAsync(&P.gscr, bytes, stream);
-        if (e != cudaSuccess) {
-            P.gscr = nullptr;
-            return cuda_err(e, "gradient scratch");
-        }
-        P.gscr_bytes = bytes;
+    if (bytes > P.gscr.bytes) {
+        scratch_put(P.gscr, stream);
+        const cudaError_t e = scratch_get(P.gscr, bytes, stream);
+        if (e != cudaSuccess) return cuda_err(e, "gradient scratch");
     }
-    cudaError_t e = cudaMemsetAsync(P.gscr, 0, bytes, stream);
+    cudaError_t e = cudaMemsetAsync(P.gscr.p, 0, bytes, stream);
     if (e != cudaSuccess) return cuda_err(e, "gradient scratch reset");
     P.gscr_mask = (uint32_t)(((uint64_t)1 << k) - 1);
     P.gscr_mul = (uint32_t)(0.6180339887498949 * (double)((uint64_t)1 << k)) | 1u;
-    A.grad = P.gscr;
+    A.grad = P.gscr.p;
     A.gmul = P.gscr_mul;
     A.gmask = P.gscr_mask;
     return HG_OK;
@@ -840,10 +826,10 @@ hg_status grad_scratch_end(hg_rays &P, int gp, void *grad, cudaStream_t stream) 
     if (n <= 0) return HG_OK;
     const unsigned blocks = (unsigned)std::min<int64_t>((n + 255) / 256, (int64_t)sm_count() * 8);
     if (gp == 0)
-        grad_unhash_kernel<double><<<blocks, 256, 0, stream>>>(n, static_cast<const double *>(P.gscr), P.gscr_mul,
+        grad_unhash_kernel<double><<<blocks, 256, 0, stream>>>(n, static_cast<const double *>(P.gscr.p), P.gscr_mul,
                                                               P.gscr_mask, static_cast<double *>(grad));
     else
-        grad_unhash_kernel<float><<<blocks, 256, 0, stream>>>(n, static_cast<const float *>(P.gscr), P.gscr_mul,
+        grad_unhash_kernel<float><<<blocks, 256, 0, stream>>>(n, static_cast<const float *>(P.gscr.p), P.gscr_mul,
                                                              P.gscr_mask, static_cast<float *>(grad));
     note_launches(1);
     cudaError_t e = cudaGetLastError();
@@ -865,18 +851,12 @@ hg_status make_staging(hg_rays &P, int prec, int64_t per_ray, cudaStream_t strea
     const size_t b_next = al((size_t)nchunks * sizeof(uint32_t)), b_sr = al((size_t)P.n * sizeof(uint32_t));
     const size_t b_ss = al((size_t)std::max<int64_t>(P.seg_cap, 1) * sizeof(uint32_t)), b_ctr = 256;
     const size_t total = b_ent + b_next + b_sr + b_ss + b_ctr;
-    if (total > P.stg_bytes) {
-        if (P.stg) cudaFreeAsync(P.stg, stream);
-        P.stg = nullptr;
-        P.stg_bytes = 0;
-        cudaError_t e = cudaMallocAsync((void **)&P.stg, total, stream);
-        if (e != cudaSuccess) {
-            P.stg = nullptr;
-            return cuda_err(e, "emission staging");
-        }
-        P.stg_bytes = total;
+    if (total > P.stg.bytes) {
+        scratch_put(P.stg, stream);
+        const cudaError_t e = scratch_get(P.stg, total, stream);
+        if (e != cudaSuccess) return cuda_err(e, "emission staging");
     }
-    unsigned char *q = P.stg;
+    unsigned char *q = static_cast<unsigned char *>(P.stg.p);
     P.stg_ent = q;
     q += b_ent;
     P.stg_next = reinterpret_cast<uint32_t *>(q);
@@ -1458,6 +1438,8 @@ extern "C" hg_status hg_rays_prepare(const hg_grid *g, int64_t n, const double *
     }
     r->g = g;
     r->n = n;
+    r->device = g->device;
+    scratch_users(r->device, 1);
     *out = r;
     return HG_OK;
 }
@@ -1709,6 +1691,7 @@ extern "C" hg_status hg_rays_gradient(hg_rays *r, double kappa, const float *w, 
 extern "C" void hg_rays_free(hg_rays *r, hg_stream stream) {
     if (!r) return;
     free_plan(*r, (cudaStream_t)stream);
+    scratch_users(r->device, -1);
     delete r;
 }
 
@@ -1744,15 +1727,16 @@ extern "C" hg_status hg_scan_offsets(int64_t n, const int32_t *count, int64_t *s
     }
     const int64_t tile = (int64_t)kScanBlock * kScanItems;
     const int64_t tiles = (n + tile - 1) / tile;
-    int64_t *sums = nullptr;
-    cudaError_t e = cudaMallocAsync((void **)&sums, (size_t)tiles * sizeof(int64_t), s);
+    Scratch scratch;
+    cudaError_t e = scratch_get(scratch, (size_t)tiles * sizeof(int64_t), s);
     if (e != cudaSuccess) return cuda_err(e, "scan scratch");
+    int64_t *sums = static_cast<int64_t *>(scratch.p);
     scan_tile_sums<<<(unsigned)tiles, kScanBlock, 0, s>>>(n, count, sums);
     scan_tile_prefix<<<1, kScanBlock, 0, s>>>(tiles, sums);
     scan_tile_apply<<<(unsigned)tiles, kScanBlock, 0, s>>>(n, count, sums, seg_off);
     note_launches(3);
     e = cudaGetLastError();
-    cudaFreeAsync(sums, s);
+    scratch_put(scratch, s);
     return e == cudaSuccess ? HG_OK : cuda_err(e, "scan launch");
 }
 
