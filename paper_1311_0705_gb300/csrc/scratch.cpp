@@ -3,46 +3,60 @@
 // The device's stream-ordered pool hands its memory back to the system whenever the host waits for the GPU, so a
 // program that waits after every call paid for mapping the next call's scratch anew: a call of 255 rays took
 // 267 us alone against 49 among others, now 82; a step of 1e6 rays with staged emission (1 GB of scratch) 4.37 ms
-// against 1.23, now 1.22.  Blocks of finished calls are therefore kept, at most kKeep bytes per device, while a grid or
-// ray plan of that device is alive, and reused.
-//   * A kept block is only given to a call on the stream that used it last (no call ever waits for another
-//     stream's work because of its scratch), and the stream waits for the event recorded at its release, so
+// against 1.23, now 1.22.  Blocks of finished calls are therefore kept, at most kKeep bytes in kBlocks blocks per
+// device, while a grid or ray plan of that device is alive, and reused.
+//   * A kept block is only given to a call on the stream that used it last, and only makes room for blocks of
+//     that stream (no call waits for another stream's work because of its scratch; what finds no room goes back
+//     to the pool, as all blocks did before).  The stream waits for the event recorded at a block's release, so
 //     that a new stream that got a destroyed one's handle is ordered too.
 //   * Under stream capture blocks come from and go to the allocator, as graph nodes: a graph's scratch is its own.
+//   * The list of kept blocks is a fixed array: nothing here allocates on the host or throws.
 //   * When an allocation fails the kept blocks are released and it is tried again.
 // (Kept blocks are freed by cudaFreeAsync throughout: after cudaFree the pool went on counting them as used.)
 #include "scratch.h"
 
 #include <mutex>
-#include <vector>
 
 namespace hg {
 namespace {
 
 constexpr size_t kKeep = (size_t)2 << 30;
 
+constexpr int kBlocks = 64;  // kept blocks of a device
+
 struct Idle {
     Scratch s;
-    int device;
     cudaStream_t stream;
 };
+// Blocks of a device, oldest first.
+struct Blocks {
+    Idle v[kBlocks];
+    int n = 0;
+    Scratch remove(int i) {
+        const Scratch s = v[i].s;
+        for (n--; i < n; i++) v[i] = v[i + 1];
+        return s;
+    }
+};
+struct Device {
+    Blocks idle;
+    size_t kept = 0;
+    int users = 0;
+};
 std::mutex g_mtx;
-std::vector<Idle> g_idle;  // oldest first
 constexpr int kDevices = 64;
-size_t g_kept[kDevices] = {};
-int g_users[kDevices] = {};
+Device g_dev[kDevices];
 
 bool capturing(cudaStream_t stream) {
     cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
     return cudaStreamIsCapturing(stream, &st) != cudaSuccess || st != cudaStreamCaptureStatusNone;
 }
 
-// Take the idle blocks of a device out of the list (under the lock).
-std::vector<Idle> take_all(int device) {
-    std::vector<Idle> out, rest;
-    for (const Idle &i : g_idle) (i.device == device ? out : rest).push_back(i);
-    g_idle.swap(rest);
-    g_kept[device] = 0;
+// Take a device's idle blocks (under the lock).
+Blocks take_all(Device &d) {
+    const Blocks out = d.idle;
+    d.idle.n = 0;
+    d.kept = 0;
     return out;
 }
 
@@ -69,18 +83,18 @@ cudaError_t scratch_get(Scratch &s, size_t bytes, cudaStream_t stream) {
     }
     {
         std::lock_guard<std::mutex> lock(g_mtx);
-        size_t best = g_idle.size();
-        for (size_t i = 0; i < g_idle.size(); i++) {
-            const Idle &c = g_idle[i];
+        Device &d = g_dev[device];
+        int best = -1;
+        for (int i = 0; i < d.idle.n; i++) {
+            const Idle &c = d.idle.v[i];
             // not a block that several smaller ones could be made of
-            if (c.device == device && c.stream == stream && c.s.bytes >= bytes && c.s.bytes / 4 <= bytes + ((size_t)1 << 20) &&
-                (best == g_idle.size() || c.s.bytes < g_idle[best].s.bytes))
+            if (c.stream == stream && c.s.bytes >= bytes && c.s.bytes / 4 <= bytes + ((size_t)1 << 20) &&
+                (best < 0 || c.s.bytes < d.idle.v[best].s.bytes))
                 best = i;
         }
-        if (best < g_idle.size()) {
-            s = g_idle[best].s;
-            g_kept[device] -= s.bytes;
-            g_idle.erase(g_idle.begin() + (std::ptrdiff_t)best);
+        if (best >= 0) {
+            s = d.idle.remove(best);
+            d.kept -= s.bytes;
         }
     }
     if (s.p) {
@@ -91,13 +105,13 @@ cudaError_t scratch_get(Scratch &s, size_t bytes, cudaStream_t stream) {
     e = cudaMallocAsync(&s.p, bytes, stream);
     if (e == cudaErrorMemoryAllocation) {
         cudaGetLastError();
-        std::vector<Idle> all;
+        Blocks all;
         {
             std::lock_guard<std::mutex> lock(g_mtx);
-            all = take_all(device);
+            all = take_all(g_dev[device]);
         }
-        for (const Idle &i : all) release_in(i.s, stream);
-        if (!all.empty()) cudaStreamSynchronize(stream);
+        for (int i = 0; i < all.n; i++) release_in(all.v[i].s, stream);
+        if (all.n > 0) cudaStreamSynchronize(stream);
         e = cudaMallocAsync(&s.p, bytes, stream);
     }
     if (e != cudaSuccess) {
@@ -115,50 +129,53 @@ cudaError_t scratch_get(Scratch &s, size_t bytes, cudaStream_t stream) {
 void scratch_put(Scratch &s, cudaStream_t stream) {
     if (!s.p) return;
     int device = -1;
-    std::vector<Scratch> drop;
+    Blocks drop;
     bool keep = s.done && !capturing(stream) && cudaGetDevice(&device) == cudaSuccess && device < kDevices &&
                 s.bytes <= kKeep && cudaEventRecord(s.done, stream) == cudaSuccess;
     if (keep) {
         std::lock_guard<std::mutex> lock(g_mtx);
-        keep = g_users[device] > 0;
+        Device &d = g_dev[device];
+        keep = d.users > 0;
         if (keep) {
-            for (size_t i = 0; i < g_idle.size() && g_kept[device] + s.bytes > kKeep;) {
-                if (g_idle[i].device != device) {
+            for (int i = 0; i < d.idle.n && (d.idle.n == kBlocks || d.kept + s.bytes > kKeep);) {
+                if (d.idle.v[i].stream != stream) {
                     i++;
                     continue;
                 }
-                drop.push_back(g_idle[i].s);
-                g_kept[device] -= g_idle[i].s.bytes;
-                g_idle.erase(g_idle.begin() + (std::ptrdiff_t)i);
+                drop.v[drop.n].s = d.idle.remove(i);
+                d.kept -= drop.v[drop.n++].s.bytes;
             }
-            g_idle.push_back({s, device, stream});
-            g_kept[device] += s.bytes;
+            keep = d.idle.n < kBlocks && d.kept + s.bytes <= kKeep;
+        }
+        if (keep) {
+            d.idle.v[d.idle.n++] = {s, stream};
+            d.kept += s.bytes;
         }
     }
     if (!keep) {
         cudaFreeAsync(s.p, stream);
         if (s.done) cudaEventDestroy(s.done);
     }
-    for (const Scratch &d : drop) release_in(d, stream);
+    for (int i = 0; i < drop.n; i++) release_in(drop.v[i].s, stream);
     s = Scratch();
 }
 
 void scratch_users(int device, int delta) {
     if (device < 0 || device >= kDevices) return;
-    std::vector<Idle> all;
+    Blocks all;
     {
         std::lock_guard<std::mutex> lock(g_mtx);
-        g_users[device] += delta;
-        if (g_users[device] <= 0) all = take_all(device);
+        g_dev[device].users += delta;
+        if (g_dev[device].users <= 0) all = take_all(g_dev[device]);
     }
-    if (all.empty()) return;
+    if (all.n == 0) return;
     int cur = 0;
     cudaGetDevice(&cur);
     if (cur != device) cudaSetDevice(device);
-    for (const Idle &i : all) {
-        cudaEventSynchronize(i.s.done);
-        cudaFreeAsync(i.s.p, 0);
-        cudaEventDestroy(i.s.done);
+    for (int i = 0; i < all.n; i++) {
+        cudaEventSynchronize(all.v[i].s.done);
+        cudaFreeAsync(all.v[i].s.p, 0);
+        cudaEventDestroy(all.v[i].s.done);
     }
     if (cur != device) cudaSetDevice(cur);
 }
