@@ -52,15 +52,16 @@ BYTES_PER_RAY = {"fp64": 48 + 8 + 4 + 1, "fp32k": 48 + 4 + 4 + 1}
 STAGE_BYTES_PER_CROSSING = {"fp64": 4 + 8, "fp32k": 4 + 4}
 STAGE_BYTES_PER_RAY = 4
 L2_FLUSH_BYTES = 512 << 20
-# what bounds the walk besides the copy bandwidth (see DESIGN, GB300-specific choices 1 and 4): random
-# gathers of 96-byte records from a 2 GB array sustained 13.2 G records/s (~1.27 TB/s) in a separate probe,
-# and FP64 add / fused multiply-add issued 16.5 G warp instructions/s (0.053 per cycle per SM) whether 32,
-# 16 or 1 lane was active, i.e. 528 G lane operations/s at full warps; per crossing the walk issues 10 FP64
-# instructions (3 wall times of 2 each, 2 fused exit-point coordinates, ds, the fused sum; under FP32-Kahan
-# the sum leaves the FP64 pipe and the FP32 cast of ds joins it)
-RANDOM_GATHER_GBS = 1.27e3
+# what bounds the walk besides the copy bandwidth: random gathers of 64-byte records from a 2 GB array
+# sustained 19.6 G records/s (1.25 TB/s) in a separate probe (96-byte records 13.2 G/s, 1.27 TB/s), and FP64
+# add / fused multiply-add issued 16.5 G warp instructions/s (0.053 per cycle per SM) whether 32, 16 or 1
+# lane was active, i.e. 528 G lane operations/s at full warps; per crossing the walk of grids with
+# single-precision bounds (all of these workloads) issues 4 FP64 instructions (2 for the time of the wall
+# that is crossed, ds, the fused sum; under FP32-Kahan the sum leaves the FP64 pipe and the FP32 cast of ds
+# joins it), the walk of other grids 10
+RANDOM_GATHER_GBS = 1.25e3
 FP64_OPS_PER_S = 528e9
-FP64_OPS_PER_CROSSING = {"fp64": 10, "fp32k": 10}
+FP64_OPS_PER_CROSSING = {"fp64": 4, "fp32k": 4}
 
 
 # ----------------------------------------------------------------------------- distributed plumbing
@@ -168,7 +169,7 @@ class ClockSampler:
 
 def kernel_source_sha() -> str:
     h = hashlib.sha256()
-    for f in ("walk.cuh", "trace.cu", "hg_internal.h"):
+    for f in ("walk.cuh", "walkf.cuh", "trace_args.cuh", "trace.cu", "tracef.cu", "hg_internal.h"):
         h.update(open(os.path.join(ROOT, "paper_1311_0705_gb300", "csrc", f), "rb").read())
     return h.hexdigest()[:16]
 
@@ -485,7 +486,7 @@ def run_ours(args):
                         note=f"{FP64_OPS_PER_CROSSING[prec]} FP64 instructions per crossing at the 528 G lane "
                              "operations/s this GPU issues with full warps bound the walk at fp64_issue_gcross_per_s, "
                              "i.e. fp64_issue_frac_of_peak "
-                             "of the copy bandwidth in algorithmic bytes; random 96-byte record gathers from "
+                             "of the copy bandwidth in algorithmic bytes; random 64-byte record gathers from "
                              "beyond L2 sustain random_gather_gbs (separate probes); L2 serves part of the records"))
 
     # the emitted cell sequences of the last step, on the host (the navigation comparison reads a sample)
@@ -513,19 +514,25 @@ def run_ours(args):
         # two sets of the tau, count and gradient buffers, so that a step never waits for the copies
         # of the step before (a set is rewritten two steps later, after the event `small` of its
         # copies); the CSR arrays are new tensors every step, kept alive for the copy stream by
-        # record_stream.
+        # record_stream.  A grid's copies also wait for the other grid's issued before them: where the
+        # link was free to serve one grid's copies of two steps first, the steps waited for the other's,
+        # and one run in six took 6.1 ms per step instead of 4.1.
         cstreams = [torch.cuda.Stream(device=dev) for _ in grids]
         hidx = {g["name"]: i for i, g in enumerate(grids)}
         for g in grids:
             g["alt"] = dict(tau=torch.empty_like(g["tau"]), nc=torch.empty_like(g["nc"]),
                             grad=torch.zeros_like(g["grad"]))
         small = [[None, None] for _ in grids]  # per grid and buffer set: the end of its small copies
+        tail = [None for _ in grids]  # per grid: the end of its copies
         cur = [0]
 
         def copy_out(g):
             i = hidx[g["name"]]
             cs = cstreams[i]
             cs.wait_stream(torch.cuda.current_stream())
+            for ev in tail[:i] + tail[i + 1:]:
+                if ev is not None:
+                    cs.wait_event(ev)
             h = hout[i]
             with torch.cuda.stream(cs):
                 for dst, src in ((h[0], g["tau"]), (h[1], g["nc"]), (h[5], g["grad"]), (h[2], g["off"])):
@@ -536,6 +543,8 @@ def run_ours(args):
                 for dst, src in ((h[3], g["cell"]), (h[4], g["ds"])):
                     src.record_stream(cs)
                     dst.copy_(src[:dst.shape[0]], non_blocking=True)
+                tail[i] = torch.cuda.Event()
+                tail[i].record(cs)
             g["off"].record_stream(cs)
 
         # the inputs of the next step are copied in on a stream of their own while the current step
@@ -558,6 +567,7 @@ def run_ours(args):
             # nsteps end-to-end steps; returns their span in ms (CUDA events on the main stream)
             for lst in [ready, done] + small:
                 lst[0] = lst[1] = None
+            tail[:] = [None for _ in grids]
             a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
             a.record(stream)
             h2d.wait_stream(stream)
@@ -838,7 +848,10 @@ def navigation_costs(H, ropes, seg_off, seg_cell, n_rays=20000):
     """Exact per-crossing costs of finding the next leaf, from the emitted cell sequences of n_rays rays:
     with neighbor lists, the position of the next leaf in the exit wall's list (records tested, tail ids
     read), or, for a list too long to store whose head misses, the descent below the wall's rope node;
-    with ropes, the nodes visited below the rope and the records tested.  Bytes: 96 per record, 4 per tail id, 16 (k-d) or 32 (octree) per node.
+    with ropes, the nodes visited below the rope and the records tested.  Bytes: 96 per record, 4 per tail
+    id, 16 (k-d) or 32 (octree) per node, i.e. the lookups of the records that any grid can have; the
+    64-byte records of grids with single-precision bounds hold the neighbor, or the step between equal
+    neighbors, or the rope node, and need one record per crossing.
     Crossings through an edge or corner (no unique shared wall) count as root descents for both."""
     node_b = 32 if H.kind == 0 else 16
     n = min(n_rays, seg_off.shape[0] - 1)
@@ -915,7 +928,8 @@ def navigation_costs(H, ropes, seg_off, seg_cell, n_rays=20000):
                 rope_to_leaf=float(to_leaf.sum() / m), rope_to_leaf_hit=float(hit_leaf.sum() / m))
     rope["bytes"] = 96 * rope["records"] + node_b * rope["nodes"]
     return dict(transitions=int(a.shape[0]), edge_or_corner=float((~face).sum() / m), lists=lists, ropes=rope,
-                bytes_note="next-leaf lookups only; every crossing also reads nothing else for navigation")
+                bytes_note="next-leaf lookups of the 96-byte records; 64-byte records: one record per crossing, "
+                           "nodes below the rope where a wall has unequal neighbors")
 
 
 def measure_navigation(hg, torch, grids, O, K, flush, stream, reps=5):
