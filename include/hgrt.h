@@ -313,7 +313,7 @@ typedef struct hg_trace_opts {
     int32_t schedule;    /* 0 = tuned or automatic; 1 = static ray stride; 2 = dynamic queue (warp-aggregated
                             counter) in input order; 3 = dynamic queue, rays with the most estimated
                             crossings first (automatic when there are fewer than 48 rays per
-                            resident thread) */
+                            resident thread; the order is left out when every ray has a thread) */
     int32_t min_blocks;  /* 0 = tuned or default (4; 3 for hg_find_interactions, whose walk needs more
                             than 64 registers); 3 or 4 resident 256-thread blocks per SM the register
                             budget of the walks of 96-byte records is cut for (80 or 64 registers; each walking
@@ -327,9 +327,12 @@ typedef struct hg_trace_opts {
 /* Path segments.  With schedule 3 (work-ordered queue), in hg_trace_rays,
  * hg_trace_rays_rho and hg_tau_gradient, a path whose estimated crossings
  * exceed max(64, A) is cut into at most 16 segments of about max(32, A/2)
- * that separate threads walk (A = estimated total / the launch's threads;
- * HG_SPLIT_FORCE: every path of more than 3, in pieces of 2, for testing).  Cuts lie at the middle of a leaf the path crosses,
- * deep inside it, so every segment follows the whole path's cell sequence:
+ * that separate threads walk (A = estimated total / the launch's threads);
+ * with schedule and split automatic and a thread for every ray, no queue is
+ * ordered and paths above max(18, 3A/4) are cut into pieces of about
+ * max(12, A/2).  HG_SPLIT_FORCE: every path of more than 3, in pieces of 2,
+ * for testing.  Cuts lie at the middle of a leaf the path crosses, deep
+ * inside it, so every segment follows the whole path's cell sequence:
  * crossing counts, statuses, emitted cells and gradients are those of the
  * unsplit walk; tau is the sum of the segments' partial sums, which differs
  * from the left-to-right sum only in the grouping of the additions (a few
