@@ -33,7 +33,10 @@
 // Whatever these bounds leave open (a few crossings in a thousand) is
 // decided by the contract's own FP64 arithmetic, as are all crossings of rays
 // whose direction components leave [2^-30, 2^30] or whose origin is far out
-// (SG_EXACT): E and eps are infinite there and every comparison fails.  A NaN
+// or, next to a wall at zero, has a component below 2^-60 (o32 = o (1 + u)
+// and a normal E would not hold down to the smallest numbers; a component
+// that is zero is exact) (SG_EXACT): E and eps are infinite there and every
+// comparison fails.  A NaN
 // fails every comparison too.  An axis with a zero direction gets i32 = 2^100
 // and E = 2^100 (bound of the position error): its wall counts as out of
 // reach unless the ray runs within that bound of it.
@@ -160,8 +163,9 @@ __device__ __forceinline__ RayStartF start_f(const RayStart &R, const double *__
     for (int a = 0; a < 3; a++) {
         const double x = o[3 * r + a], k = d[3 * r + a];
         S.o[a] = dzero(x) ? 0.0 : x;
-        const float m = fabsf(near_float(k));
-        exact = exact || !(fabsf(near_float(x)) <= 0x1p20f) || !(dzero(k) || (m >= 0x1p-30f && m <= 0x1p30f));
+        const float m = fabsf(near_float(k)), mo = fabsf(near_float(x));
+        exact = exact || !(dzero(x) || (mo >= 0x1p-60f && mo <= 0x1p20f)) ||
+                !(dzero(k) || (m >= 0x1p-30f && m <= 0x1p30f));
     }
     S.sg = R.sg | (exact ? SG_EXACT : 0u);
     return S;
