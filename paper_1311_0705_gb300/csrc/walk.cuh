@@ -24,6 +24,7 @@
 #include <cstddef>
 
 #include "hg_internal.h"
+#include "plan_rules.h"
 
 namespace hg {
 
@@ -250,24 +251,22 @@ __device__ __forceinline__ void stage_lattice(const DevGrid &G, float *lat) {
 constexpr int kWorkSamples = 16;
 __device__ __forceinline__ float work_estimate(const DevGrid &G, const float *lat, const float *o, const float *k,
                                                float t0, float t1) {
-    static_assert(kWorkN == 16, "cells are taken from the low four bits");
+    static_assert(kWorkN == 16, "lattice_cell is made for 16 cells");
     if (!(t1 > t0)) return 0.0f;
-    // cell number = floor of the lattice coordinate, read off the low mantissa bits of (coordinate - 1/2) + 2^23
-    // rounded to a whole number (a coordinate on a cell's edge may count for either side)
     const float dt = (t1 - t0) * (1.0f / (float)kWorkSamples);
     float p[3], dp[3];
 #pragma unroll
     for (int a = 0; a < 3; a++) {
-        const float sc = __fdividef((float)kWorkN, G.fhi[a] - G.flo[a]);
+        const float sc = __fdividef((float)kWorkN * kLatticeScale, G.fhi[a] - G.flo[a]);
         dp[a] = k[a] * dt * sc;
-        p[a] = (o[a] + k[a] * t0 - G.flo[a]) * sc - 0.5f + 0.5f * dp[a];
+        p[a] = (o[a] + k[a] * t0 - G.flo[a]) * sc - kLatticeShift + 0.5f * dp[a];
     }
     float e = 0.0f;
 #pragma unroll
     for (int j = 0; j < kWorkSamples; j++) {
-        const uint32_t x = __float_as_uint(__fmaf_rn((float)j, dp[0], p[0]) + 0x1p23f) & 15u;
-        const uint32_t y = __float_as_uint(__fmaf_rn((float)j, dp[1], p[1]) + 0x1p23f) & 15u;
-        const uint32_t z = __float_as_uint(__fmaf_rn((float)j, dp[2], p[2]) + 0x1p23f) & 15u;
+        const uint32_t x = lattice_cell(__fmaf_rn((float)j, dp[0], p[0]));
+        const uint32_t y = lattice_cell(__fmaf_rn((float)j, dp[1], p[1]));
+        const uint32_t z = lattice_cell(__fmaf_rn((float)j, dp[2], p[2]));
         e += lat[x | y << 4 | z << 8];
     }
     return e * dt;
