@@ -26,4 +26,17 @@ HG_HOST_DEVICE uint32_t lattice_cell(float p) {
     return b & 15u;
 }
 
+// Whether cut c of a path is made: candidates 0 .. c in path order by their numbers, at times t (minus infinity where there is
+// none) in leaves `leaf`.  A cut is made when it lies later than the last one made and in another leaf (the path
+// starts at t0 in leaf0).
+HG_HOST_DEVICE bool cut_made(const float *t, const int32_t *leaf, int c, float t0, int32_t leaf0) {
+    bool made = false;
+    for (int j = 0; j <= c; j++) {
+        made = t[j] > t0 && leaf[j] != leaf0;
+        t0 = made ? t[j] : t0;
+        leaf0 = made ? leaf[j] : leaf0;
+    }
+    return made;
+}
+
 }  // namespace hg

@@ -134,7 +134,7 @@ struct SplitRec {
 // end of the work-ordered queue, or over all rays when there is none: the
 // lanes sample the work lattice at 32 points of the path and sum them
 // (a prefix sum), lane j places cut j where the sum reaches (j + 1) / K
-// of the total (descent and depth test), and the accepted cuts are those of
+// of the total (descent and depth test), and the cuts made (cut_made) are those of
 // increasing t_c in distinct leaves, in path order.  Segment slots are
 // taken with one atomic per ray; their count is bounded (sum over split
 // rays of ceil(w/W) <= total/W + total/threshold <= 3.4 T, or 16 n when
@@ -158,6 +158,7 @@ __global__ void __launch_bounds__(256) split_kernel(const DevGrid G, int64_t n, 
     Start *starts = static_cast<Start *>(starts_v);
     __shared__ int32_t s_leaf[kPlanRays][kMaxSegs];
     __shared__ long long s_key[kPlanRays][kMaxSegs];
+    __shared__ float s_time[kPlanRays][kMaxSegs];
     __shared__ long long s_ncand;
     __shared__ __align__(16) float lat[kWorkN * kWorkN * kWorkN];
     extern __shared__ __align__(16) unsigned char snodes[];  // the top n_smem nodes, where the descents start
@@ -292,14 +293,12 @@ __global__ void __launch_bounds__(256) split_kernel(const DevGrid G, int64_t n, 
                 }
             }
         }
+        // cuts are made in path order, each later than the one made before and in another leaf
+        s_time[slot][lane] = ok ? tc : -CUDART_INF_F;
+        s_leaf[slot][lane] = Lid;
         __syncwarp(half);
-        // accept cuts in path order: later than the cut before and in another leaf (the leaves a path crosses
-        // do not recur, so that comparing with the cut before, accepted or not, is enough)
-        const unsigned oks = (__ballot_sync(half, ok) & half) >> (threadIdx.x & 16);
-        const int before = 31 - __clz(oks & ((1u << lane) - 1u));  // -1: none
-        const float t_prev = __shfl_sync(half, tc, before < 0 ? 0 : before, 16);
-        const int32_t l_prev = __shfl_sync(half, Lid, before < 0 ? 0 : before, 16);
-        const bool take = ok && tc > (before < 0 ? ts : t_prev) && Lid != (before < 0 ? R.cur : l_prev);
+        const bool take = ok && cut_made(s_time[slot], s_leaf[slot], lane, ts, R.cur);
+        __syncwarp(half);
         const unsigned cuts = (__ballot_sync(half, take) & half) >> (threadIdx.x & 16);
         const int ncut = __popc(cuts);
         if (ncut == 0) continue;

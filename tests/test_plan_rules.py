@@ -13,6 +13,9 @@ SRC = r"""
 extern "C" void cells(int n, const float *x, uint32_t *out) {
     for (int i = 0; i < n; i++) out[i] = hg::lattice_cell(x[i] * hg::kLatticeScale - hg::kLatticeShift);
 }
+extern "C" void cuts(int n, const float *t, const int32_t *leaf, float t0, int32_t leaf0, uint8_t *out) {
+    for (int c = 0; c < n; c++) out[c] = hg::cut_made(t, leaf, c, t0, leaf0);
+}
 """
 
 
@@ -47,3 +50,27 @@ def test_any_coordinate_gives_a_cell(rules):
     out = np.empty(len(x), np.uint32)
     rules.cells(len(x), _p(x), _p(out))
     assert (out < 16).all()
+
+
+def _cuts(rules, t, leaf, t0, leaf0):
+    t, leaf, out = np.array(t, np.float32), np.array(leaf, np.int32), np.zeros(len(t), np.uint8)
+    rules.cuts(len(t), _p(t), _p(leaf), ctypes.c_float(t0), leaf0, _p(out))
+    return [j for j in range(len(t)) if out[j]]
+
+
+def test_cuts_follow_each_other(rules):
+    none = -np.inf
+    assert _cuts(rules, [1, 2, 3], [5, 6, 7], 0.0, 4) == [0, 1, 2]
+    assert _cuts(rules, [1, none, 3], [5, -1, 7], 0.0, 4) == [0, 2]
+    assert _cuts(rules, [none, none], [-1, -1], 0.0, 4) == []
+    assert _cuts(rules, [1, 1, 2], [5, 5, 6], 0.0, 4) == [0, 2]  # the same leaf twice
+    assert _cuts(rules, [1, 2], [4, 6], 0.0, 4) == [1]           # the first leaf
+    # a time out of order, and one between: segments must not run backwards
+    assert _cuts(rules, [1, 3, 2, 2.5, 4], [5, 7, 6, 8, 9], 0.0, 4) == [0, 1, 4]
+    rng = np.random.default_rng(1)
+    for _ in range(200):
+        t, leaf = rng.integers(0, 20, 15).astype(float), rng.integers(0, 9, 15)
+        t[rng.random(15) < 0.2] = none
+        made = _cuts(rules, t, leaf, 1.0, 3)
+        assert (np.diff([1.0] + list(t[made])) > 0).all()
+        assert (np.diff([3] + list(leaf[made])) != 0).all()
