@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cmath>
 #include <vector>
 
 #include "hg_internal.h"
@@ -67,7 +68,7 @@ __device__ double rho_true(const DevModel &m, double x, double y, double z) {
 // One evaluation of the disk's density through the CUDA math library is two divisions, a square root and an
 // exponential: about 50 instructions of the FP64 pipe, which issues one warp instruction per 19 cycles and SM and is
 // what both kernels below wait for.  With reciprocals prepared per launch or path, and the two functions
-// written for the arguments that occur (positive normal numbers), it is 20 in the quadrature and 25 for points.
+// written for the arguments that occur (positive normal numbers), it is 22 in the quadrature and 25 for points.
 
 constexpr double kExpLimit = 690.0;  // exp_neg's largest argument
 
@@ -395,44 +396,56 @@ __global__ void model_tau_kernel(const DevModel m, int64_t n, const double *__re
 // The bound is the FP64 pipe, which a warp instruction holds for 19 cycles whatever its active lanes.  With a
 // path per thread a warp lasted as long as its longest path (17.6 rule evaluations per path on average, 45
 // for the longest of 32: the pipe did 2.5 times the work), and an evaluation cost ~100 FP64 instructions.
-// In units of the scale lengths, with u = t - t0 the parameter from the closest approach to the axis, the
-// exponent along a path is sqrt(A u^2 + D2) + |oz + kz t|: with the functions above 20 FP64 instructions, 24
-// with the rule's sums.  1e5 paths between random points of the cube: 12.4 ms -> 1.35 ms
-// (24 instructions for 26.5e6 evaluations: 1.2 ms).
+// A density is evaluated at the point o + k t, with the functions above 22 FP64 instructions and 26 with the rule's sums.  (In units of
+// the scale lengths from the closest approach to the axis, sqrt(A u^2 + D2) + |oz + kz t|, it was two fewer, but A and D2 were
+// wrong where the square of a nearly vertical path's horizontal part underflows, and their roundings, the same
+// all along the path, do not average out.)
 //
 // A pool that is nearly full is worked down one interval at a time, depth first (an interval needs at most
 // kMaxDepth entries beyond its own).  The sums of a path are added in pool order: the same terms as in path_integral,
 // in another order.
 constexpr int kTauWarps = 8, kPool = 256, kSlots = 64, kMaxDepth = 60;
-// A path in units of the scale lengths.
+// The scale lengths as the kernel uses them.
+struct DiskScale {
+    double unit;    // power of two: h_R unit is between 1 and 2
+    double rR, rz;  // 1 / (h_R unit), 1 / h_z
+};
+DiskScale disk_scale(const DevModel &m) {
+    DiskScale q;
+    int e;
+    frexp(m.p[1], &e);
+    q.unit = ldexp(1.0, 1 - e);
+    q.rR = 1.0 / (m.p[1] * q.unit);
+    q.rz = 1.0 / m.p[2];
+    return q;
+}
+// A path, its horizontal part times DiskScale's unit (exact).
 struct DiskPath {
-    double t0, A, D2, oz, kz;
+    double o[3], k[3];
     bool ordinary;  // something to integrate, the exponent in exp_neg's range all along
-    __device__ __forceinline__ DiskPath(const DevModel &m, const double *o, const double *k, double L) {
-        const double kk = k[0] * k[0] + k[1] * k[1];
-        const double cr = o[0] * k[1] - o[1] * k[0];
-        const double h2 = m.p[1] * m.p[1];
-        t0 = kk > 0.0 ? -(o[0] * k[0] + o[1] * k[1]) / kk : 0.0;
-        A = kk / h2;
-        D2 = (kk > 0.0 ? cr * cr / kk : o[0] * o[0] + o[1] * o[1]) / h2;
-        oz = o[2] / m.p[2];
-        kz = k[2] / m.p[2];
-        const double far = fmax(fabs(t0), fabs(L - t0));  // the exponent is convex: largest at an end
-        const double s = sqrt(A * far * far + D2) + fmax(fabs(oz), fabs(oz + kz * L));
-        ordinary = L > 0.0 && s <= kExpLimit;
-        D2 += 0x1p-100;  // a path through the axis: keeps the root's argument normal
+    __device__ __forceinline__ DiskPath(const DiskScale &q, const double *oo, const double *kk, double L) {
+#pragma unroll
+        for (int a = 0; a < 3; a++) {
+            o[a] = a < 2 ? oo[a] * q.unit : oo[a];
+            k[a] = a < 2 ? kk[a] * q.unit : kk[a];
+        }
+        auto s = [&](double t) {
+            const double x = fma(k[0], t, o[0]), y = fma(k[1], t, o[1]), z = fma(k[2], t, o[2]);
+            return sqrt(x * x + y * y) * q.rR + fabs(z) * q.rz;
+        };
+        ordinary = L > 0.0 && s(0.0) <= kExpLimit && s(L) <= kExpLimit;  // the exponent is convex: largest at an end
     }
 };
 struct TauWarp {
     double a[kPool], b[kPool];                       // intervals
-    double t0[kSlots], A[kSlots], D2[kSlots], oz[kSlots], kz[kSlots];  // paths under way
+    double o[3][kSlots], k[3][kSlots];               // paths under way (DiskPath)
     double acc[kSlots];
     long long path[kSlots];
     int left[kSlots];                                // intervals of the path not yet added (0: the slot is free)
     int meta[kPool];                                 // slot | depth << 8
 };
 
-__global__ void __launch_bounds__(32 * kTauWarps, 2) disk_tau_kernel(const DevModel m, int64_t n, int64_t share,
+__global__ void __launch_bounds__(32 * kTauWarps, 2) disk_tau_kernel(const DevModel m, const DiskScale q, int64_t n, int64_t share,
                                                                   const double *__restrict__ O,
                                                                   const double *__restrict__ K,
                                                                   const double *__restrict__ len, double kappa,
@@ -475,11 +488,13 @@ __global__ void __launch_bounds__(32 * kTauWarps, 2) disk_tau_kernel(const DevMo
                 const double o[3] = {O[3 * i], O[3 * i + 1], O[3 * i + 2]};
                 const double k[3] = {K[3 * i], K[3 * i + 1], K[3 * i + 2]};
                 const double L = len[i];
-                const DiskPath P(m, o, k, L);
+                const DiskPath P(q, o, k, L);
                 if (!P.ordinary) {
                     s_other = 1;
                 } else {
-                    double c1 = P.t0, c2 = k[2] != 0.0 ? -o[2] / k[2] : 0.0;
+                    // pieces between the closest approach to the axis and the midplane
+                    const double kk = k[0] * k[0] + k[1] * k[1];
+                    double c1 = kk > 0.0 ? -(o[0] * k[0] + o[1] * k[1]) / kk : 0.0, c2 = k[2] != 0.0 ? -o[2] / k[2] : 0.0;
                     if (c2 < c1) {
                         const double c = c1;
                         c1 = c2;
@@ -489,11 +504,11 @@ __global__ void __launch_bounds__(32 * kTauWarps, 2) disk_tau_kernel(const DevMo
                     if (c1 > 0.0 && c1 < L) cut[++pieces] = c1;
                     if (c2 > 0.0 && c2 < L && c2 > cut[pieces]) cut[++pieces] = c2;
                     cut[++pieces] = L;
-                    W.t0[slot] = P.t0;
-                    W.A[slot] = P.A;
-                    W.D2[slot] = P.D2;
-                    W.oz[slot] = P.oz;
-                    W.kz[slot] = P.kz;
+#pragma unroll
+                    for (int a = 0; a < 3; a++) {
+                        W.o[a][slot] = P.o[a];
+                        W.k[a][slot] = P.k[a];
+                    }
                     W.acc[slot] = 0.0;
                     W.path[slot] = i;
                     W.left[slot] = pieces;
@@ -525,10 +540,12 @@ __global__ void __launch_bounds__(32 * kTauWarps, 2) disk_tau_kernel(const DevMo
         const int at = size - 1 - (on ? lane : 0);
         const double x0 = W.a[at], x1 = W.b[at];
         const int slot = W.meta[at] & 255, depth = W.meta[at] >> 8;
-        const double t0 = W.t0[slot], A = W.A[slot], D2 = W.D2[slot], oz = W.oz[slot], kz = W.kz[slot];
+        const double ox = W.o[0][slot], oy = W.o[1][slot], oz = W.o[2][slot];
+        const double kx = W.k[0][slot], ky = W.k[1][slot], kz = W.k[2][slot];
         auto f = [&](double t) {
-            const double u = t - t0;
-            return exp_neg<false>(sqrt_pos(fma(A * u, u, D2)) + fabs(fma(kz, t, oz)), tab);
+            const double x = fma(kx, t, ox), y = fma(ky, t, oy), z = fabs(fma(kz, t, oz));
+            const double R = sqrt_pos(fma(x, x, fma(y, y, 0x1p-118)));  // (on the axis: a normal argument)
+            return exp_neg<false>(fma(R, q.rR, z * q.rz), tab);
         };
         const double c = 0.5 * (x0 + x1), h = 0.5 * (x1 - x0);
         const double fc = f(c);
@@ -567,7 +584,7 @@ __global__ void __launch_bounds__(32 * kTauWarps, 2) disk_tau_kernel(const DevMo
         const int64_t i = first + j;
         const double o[3] = {O[3 * i], O[3 * i + 1], O[3 * i + 2]};
         const double k[3] = {K[3 * i], K[3 * i + 1], K[3 * i + 2]};
-        if (!DiskPath(m, o, k, len[i]).ordinary) tau[i] = kappa * path_integral(m, o, k, len[i], rtol);
+        if (!DiskPath(q, o, k, len[i]).ordinary) tau[i] = kappa * path_integral(m, o, k, len[i], rtol);
     }
 }
 
@@ -703,7 +720,7 @@ extern "C" hg_status hg_model_tau(const hg_dmodel *m, int64_t n, const double *o
         if (e != cudaSuccess) return cuda_err(e, "model tau shared memory");
         const int64_t blocks = std::min<int64_t>((n + kTauWarps - 1) / kTauWarps, (int64_t)sm_count() * 2);
         const int64_t share = (n + blocks - 1) / blocks;
-        disk_tau_kernel<<<(unsigned)blocks, 32 * kTauWarps, smem, (cudaStream_t)stream>>>(m->m, n, share, o, d, len,
+        disk_tau_kernel<<<(unsigned)blocks, 32 * kTauWarps, smem, (cudaStream_t)stream>>>(m->m, disk_scale(m->m), n, share, o, d, len,
                                                                                        kappa, rtol, tau);
     } else {
         const int block = 128;
