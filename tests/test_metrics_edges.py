@@ -36,3 +36,31 @@ def test_quadrature_of_nearly_vertical_paths(hg, h):
         k[2, 2] = -1.0
         L = np.array([1.0, 0.7, 0.9, 0.2])
         np.testing.assert_allclose(_tau(hg, model, o, k, L), oracle.tau_true(model, o, k, L, kappa=1.7), rtol=1e-9)
+
+
+@pytest.mark.parametrize("disk", [(1.0, 0.25, 0.03), (1.0, 0.1, 0.3)], ids=lambda d: "-".join(map(str, d)))
+def test_quadrature_rounds_no_worse_than_the_oracle(hg, disk):
+    # In a plane through the axis the exponent is linear between the cuts: closed form, in extended precision.  Both
+    # sides integrate the same intervals; 1.1 covers the other exponential and order of additions (the mean of 4000
+    # errors is known to 2 %)
+    rho_c, h_R, h_z = disk
+    model = synth.make_disk(rho_c=rho_c, h_R=h_R, h_z=h_z)
+    rng = np.random.default_rng(5)
+    n = 4000
+    a, b = rng.uniform(-1, 1, (n, 3)), rng.uniform(-1, 1, (n, 3))
+    a[:, 1] = b[:, 1] = 0.0
+    L = np.linalg.norm(b - a, axis=1)
+    k = (b - a) / L[:, None]
+    ld = np.longdouble
+    o, d, end = a.astype(ld), k.astype(ld), L.astype(ld)
+    cut = np.sort(np.clip(np.stack([-o[:, 0] / d[:, 0], -o[:, 2] / d[:, 2]], 1), 0, end[:, None]), axis=1)
+    edge = np.concatenate([np.zeros((n, 1), ld), cut, end[:, None]], axis=1)
+    s = lambda t: np.abs(o[:, 0] + d[:, 0] * t) / ld(h_R) + np.abs(o[:, 2] + d[:, 2] * t) / ld(h_z)
+    tau = np.zeros(n, ld)
+    for j in range(3):
+        t0, t1 = edge[:, j], edge[:, j + 1]
+        s0, ds = s(t0), s(t1) - s(t0)
+        tau += np.where(t1 > t0, -np.exp(-s0) * np.expm1(-ds) * (t1 - t0) / np.where(ds == 0, 1, ds), 0)
+    tau *= ld(rho_c) * ld(1.7)
+    error = lambda x: float(np.mean(np.abs(x.astype(ld) - tau) / tau))
+    assert error(_tau(hg, model, a, k, L)) <= 1.1 * error(oracle.tau_true(model, a, k, L, kappa=1.7))
