@@ -64,3 +64,14 @@ def test_quadrature_rounds_no_worse_than_the_oracle(hg, disk):
     tau *= ld(rho_c) * ld(1.7)
     error = lambda x: float(np.mean(np.abs(x.astype(ld) - tau) / tau))
     assert error(_tau(hg, model, a, k, L)) <= 1.1 * error(oracle.tau_true(model, a, k, L, kappa=1.7))
+
+
+@pytest.mark.parametrize("n", [1, 9, 300, 2433, 500_000])
+def test_quadrature_repeats_itself(hg, n):
+    model = synth.make_disk()
+    o, k, L = synth.endpoint_paths(3, n)
+    dm, args = hg.load_model(model), (_t(o), _t(k), _t(L))
+    first = hg.model_tau(dm, *args)
+    assert bool((first > 0).all())
+    for _ in range(5):
+        assert torch.equal(hg.model_tau(dm, *args), first)
