@@ -75,3 +75,14 @@ def test_quadrature_repeats_itself(hg, n):
     assert bool((first > 0).all())
     for _ in range(5):
         assert torch.equal(hg.model_tau(dm, *args), first)
+
+
+def test_densities_are_those_of_the_cuda_functions(hg):
+    # with y = 0 the radius is |x| whatever its rounding: torch's division and exponential, bit for bit
+    model = synth.make_disk()
+    p = _t(synth.sample_points(6, 200_000))
+    p[:, 1] = 0.0
+    p[100_000:, 2] *= 0.1
+    h_R, h_z = (torch.full_like(p[:, 0], float(model.params[j])) for j in (1, 2))
+    ref = torch.exp(-(p[:, 0].abs() / h_R + p[:, 2].abs() / h_z))
+    assert torch.equal(hg.model_density(hg.load_model(model), p), ref)
