@@ -617,10 +617,11 @@ __global__ void __launch_bounds__(kStatBlock) diff_partial(int64_t n, const doub
     for (int64_t i = (int64_t)blockIdx.x * kStatBlock + threadIdx.x; i < n; i += 4 * step) {
         double x[4];
 #pragma unroll
-        for (int j = 0; j < 4; j++) x[j] = i + j * step < n ? a[i + j * step] - b[i + j * step] : mu;
+        for (int j = 0; j < 4; j++) x[j] = i + j * step < n ? a[i + j * step] - b[i + j * step] : 0.0;
 #pragma unroll
         for (int j = 0; j < 4; j++) {
-            const double y = x[j] - mu;
+            // (past the end: nothing, whatever the mean is)
+            const double y = !SECOND || i + j * step < n ? x[j] - mu : 0.0;
             s[j] = SECOND ? fma(y, y, s[j]) : s[j] + x[j];
         }
     }

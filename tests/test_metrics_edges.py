@@ -86,3 +86,10 @@ def test_densities_are_those_of_the_cuda_functions(hg):
     h_R, h_z = (torch.full_like(p[:, 0], float(model.params[j])) for j in (1, 2))
     ref = torch.exp(-(p[:, 0].abs() / h_R + p[:, 2].abs() / h_z))
     assert torch.equal(hg.model_density(hg.load_model(model), p), ref)
+
+
+@pytest.mark.parametrize("n", [2, 5, 1023])
+def test_statistics_whose_sums_overflow(hg, n):
+    a = np.full(n, 1.7e308)
+    out = hg.diff_stats(_t(a), _t(np.zeros(n))).cpu().numpy()
+    np.testing.assert_array_equal(out, [n, np.inf, np.inf])
