@@ -47,10 +47,23 @@ std::mutex g_mtx;
 constexpr int kDevices = 64;
 Device g_dev[kDevices];
 
+// (A failed query leaves an error behind that the next launch's check would take for its own: cleared, here and below.)
+bool ok(cudaError_t e) {
+    if (e != cudaSuccess) cudaGetLastError();
+    return e == cudaSuccess;
+}
+
 bool capturing(cudaStream_t stream) {
     cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-    return cudaStreamIsCapturing(stream, &st) != cudaSuccess || st != cudaStreamCaptureStatusNone;
+    return !ok(cudaStreamIsCapturing(stream, &st)) || st != cudaStreamCaptureStatusNone;
 }
+
+// Queries and waits inside do not break a capture that another thread has under way.
+struct RelaxedCapture {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
 
 // Take a device's idle blocks (under the lock).
 Blocks take_all(Device &d) {
@@ -78,7 +91,7 @@ cudaError_t scratch_get(Scratch &s, size_t bytes, cudaStream_t stream) {
     if (device >= kDevices || capturing(stream)) {
         e = cudaMallocAsync(&s.p, bytes, stream);
         s.bytes = e == cudaSuccess ? bytes : 0;
-        if (e != cudaSuccess) s.p = nullptr;
+        if (!ok(e)) s.p = nullptr;
         return e;
     }
     {
@@ -99,7 +112,7 @@ cudaError_t scratch_get(Scratch &s, size_t bytes, cudaStream_t stream) {
     }
     if (s.p) {
         e = cudaStreamWaitEvent(stream, s.done, 0);
-        if (e != cudaSuccess) scratch_put(s, stream);
+        if (!ok(e)) scratch_put(s, stream);
         return e;
     }
     e = cudaMallocAsync(&s.p, bytes, stream);
@@ -111,18 +124,18 @@ cudaError_t scratch_get(Scratch &s, size_t bytes, cudaStream_t stream) {
             all = take_all(g_dev[device]);
         }
         for (int i = 0; i < all.n; i++) release_in(all.v[i].s, stream);
-        if (all.n > 0) cudaStreamSynchronize(stream);
+        if (all.n > 0) {
+            const RelaxedCapture relaxed;
+            cudaStreamSynchronize(stream);
+        }
         e = cudaMallocAsync(&s.p, bytes, stream);
     }
-    if (e != cudaSuccess) {
+    if (!ok(e)) {
         s = Scratch();
         return e;
     }
     s.bytes = bytes;
-    if (cudaEventCreateWithFlags(&s.done, cudaEventDisableTiming) != cudaSuccess) {
-        cudaGetLastError();
-        s.done = nullptr;  // not kept, then
-    }
+    if (!ok(cudaEventCreateWithFlags(&s.done, cudaEventDisableTiming))) s.done = nullptr;  // not kept, then
     return cudaSuccess;
 }
 
@@ -131,14 +144,15 @@ void scratch_put(Scratch &s, cudaStream_t stream) {
     int device = -1;
     Blocks drop;
     bool keep = s.done && !capturing(stream) && cudaGetDevice(&device) == cudaSuccess && device < kDevices &&
-                s.bytes <= kKeep && cudaEventRecord(s.done, stream) == cudaSuccess;
+                s.bytes <= kKeep && ok(cudaEventRecord(s.done, stream));
     if (keep) {
         std::lock_guard<std::mutex> lock(g_mtx);
         Device &d = g_dev[device];
         keep = d.users > 0;
         if (keep) {
             for (int i = 0; i < d.idle.n && (d.idle.n == kBlocks || d.kept + s.bytes > kKeep);) {
-                if (d.idle.v[i].stream != stream) {
+                const Idle &c = d.idle.v[i];
+                if (c.stream != stream) {
                     i++;
                     continue;
                 }
@@ -172,6 +186,7 @@ void scratch_users(int device, int delta) {
     int cur = 0;
     cudaGetDevice(&cur);
     if (cur != device) cudaSetDevice(device);
+    const RelaxedCapture relaxed;
     for (int i = 0; i < all.n; i++) {
         cudaEventSynchronize(all.v[i].s.done);
         cudaFreeAsync(all.v[i].s.p, 0);
