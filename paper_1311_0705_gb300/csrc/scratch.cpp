@@ -5,9 +5,11 @@
 // 267 us alone against 49 among others, now 82; a step of 1e6 rays with staged emission (1 GB of scratch) 4.37 ms
 // against 1.23, now 1.22.  Blocks of finished calls are therefore kept, at most kKeep bytes in kBlocks blocks per
 // device, while a grid or ray plan of that device is alive, and reused.
-//   * A kept block is only given to a call on the stream that used it last, and only makes room for blocks of
-//     that stream (no call waits for another stream's work because of its scratch; what finds no room goes back
-//     to the pool, as all blocks did before).  The stream waits for the event recorded at a block's release, so
+//   * A kept block is only given to a call on the stream that used it last.  It makes room for blocks of
+//     that stream, and for those of others when it was not used during the last kStale releases and its work
+//     has ended (a stream at rest, or destroyed): no call waits for another stream's work because of its scratch, and
+//     streams that take turns do not displace each other's blocks.  What finds no room goes back to the
+//     pool, as all blocks did before.  The stream waits for the event recorded at a block's release, so
 //     that a new stream that got a destroyed one's handle is ordered too.
 //   * Under stream capture blocks come from and go to the allocator, as graph nodes: a graph's scratch is its own.
 //   * The list of kept blocks is a fixed array: nothing here allocates on the host or throws.
@@ -15,6 +17,7 @@
 // (Kept blocks are freed by cudaFreeAsync throughout: after cudaFree the pool went on counting them as used.)
 #include "scratch.h"
 
+#include <cstdint>
 #include <mutex>
 
 namespace hg {
@@ -23,10 +26,12 @@ namespace {
 constexpr size_t kKeep = (size_t)2 << 30;
 
 constexpr int kBlocks = 64;  // kept blocks of a device
+constexpr int kStale = 128;  // releases (some tens of calls)
 
 struct Idle {
     Scratch s;
     cudaStream_t stream;
+    uint64_t turn;  // the device's count of releases when it came
 };
 // Blocks of a device, oldest first.
 struct Blocks {
@@ -41,6 +46,7 @@ struct Blocks {
 struct Device {
     Blocks idle;
     size_t kept = 0;
+    uint64_t turn = 0;  // blocks released so far
     int users = 0;
 };
 std::mutex g_mtx;
@@ -64,6 +70,12 @@ struct RelaxedCapture {
     RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
     ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
 };
+
+// Whether the work of a block's last use has ended.
+bool ended(const Scratch &s) {
+    const RelaxedCapture relaxed;
+    return ok(cudaEventQuery(s.done));
+}
 
 // Take a device's idle blocks (under the lock).
 Blocks take_all(Device &d) {
@@ -150,9 +162,10 @@ void scratch_put(Scratch &s, cudaStream_t stream) {
         Device &d = g_dev[device];
         keep = d.users > 0;
         if (keep) {
+            d.turn++;
             for (int i = 0; i < d.idle.n && (d.idle.n == kBlocks || d.kept + s.bytes > kKeep);) {
                 const Idle &c = d.idle.v[i];
-                if (c.stream != stream) {
+                if (c.stream != stream && !(d.turn - c.turn > kStale && ended(c.s))) {
                     i++;
                     continue;
                 }
@@ -162,7 +175,7 @@ void scratch_put(Scratch &s, cudaStream_t stream) {
             keep = d.idle.n < kBlocks && d.kept + s.bytes <= kKeep;
         }
         if (keep) {
-            d.idle.v[d.idle.n++] = {s, stream};
+            d.idle.v[d.idle.n++] = {s, stream, d.turn};
             d.kept += s.bytes;
         }
     }

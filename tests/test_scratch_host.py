@@ -155,6 +155,23 @@ def test_no_more_than_two_gibibytes_or_64_blocks_are_kept(fake):
     assert fake.call(3000 * MB, 3) and fake.lib.t_used() <= 2048 * MB  # larger than all that is kept
 
 
+@pytest.mark.parametrize("size,blocks", [(1000 * MB, 2), (1000, 64)], ids=["bytes", "count"])
+def test_blocks_of_a_stream_at_rest_make_room(fake, size, blocks):
+    held = [fake.get(size, 1)[1] for _ in range(blocks)]
+    for p in held:
+        fake.lib.t_put(p, 1)
+    # the stream works still: its blocks stay, whatever others do
+    for _ in range(300):
+        fake.call(size, 2)
+    assert fake.lib.t_blocks() == blocks and not fake.reused(size, 2)
+    # at rest: others' blocks take their place, in time
+    fake.lib.t_rest(1)
+    for _ in range(300):
+        fake.call(size, 2)
+    assert fake.reused(size, 2)
+    assert fake.lib.t_used() <= 2048 * MB
+
+
 def test_streams_in_turn_do_not_displace_each_other(fake):
     # two streams that are waited for after every call, with more scratch than is kept for both: one goes on with its own
     first = fake.call(1500 * MB, 1)
