@@ -16,7 +16,8 @@
  *     and released on it before the call returns; while a grid or ray plan
  *     of the device is alive, up to 2 GiB per device of released scratch is
  *     kept for later calls on the same stream (not under stream capture:
- *     a graph's scratch is its own), and freed with the last of them.
+ *     a graph's scratch is its own), and freed with the last of them, when
+ *     an allocation of this library fails, or by hg_release_scratch.
  *   - Per-ray problems never abort a launch: they are reported as bit
  *     flags (HG_RAY_*) in the optional per-ray status array.
  *   - hg_last_error() returns a message for the calling thread's last
@@ -549,6 +550,13 @@ void hg_batch_free(hg_batch *b);
 hg_status hg_batch_trace(hg_batch *b, const double *o, const double *d, const double *s_max, double kappa,
                          const hg_trace_opts *opts, void *tau, int32_t *ncross, uint8_t *ray_status,
                          hg_stream stream);
+
+/* ------------------------------------------------------------------------ kept scratch
+ * Give the current device's kept scratch (at most 2 GiB, see above) back to
+ * the system: for a program whose own allocator has run out of memory.  Waits
+ * until the calls that used it have ended; scratch of calls under way and of
+ * live ray plans is not touched, and later calls keep theirs as before. */
+hg_status hg_release_scratch(void);
 
 /* ------------------------------------------------------------------------ autotuner
  * Time candidate launch configurations (threads per block, shared-memory

@@ -140,6 +140,7 @@ _SIGS = {
     "hg_batch_free": (None, [_V]),
     "hg_batch_trace": (_S, [_V, _V, _V, _V, C.c_double, C.POINTER(TraceOpts), _V, _V, _V, _V]),
     "hg_autotune": (_S, [_V, _I64, _V, _V, C.c_int32, C.POINTER(TraceOpts), C.POINTER(C.c_float), _V]),
+    "hg_release_scratch": (_S, []),
     "hg_status_str": (C.c_char_p, [_S]),
     "hg_last_error": (C.c_char_p, []),
     "hg_version": (C.c_int32, []),
@@ -889,6 +890,11 @@ class Batch:
         if h:
             _lib.hg_batch_free(h)
             self._h = None
+
+
+def release_scratch():
+    """Give the current device's kept scratch (at most 2 GiB) back to the system (hg_release_scratch)."""
+    _check(_lib.hg_release_scratch(), "hg_release_scratch")
 
 
 def autotune(grid: Grid, o, d, precision="fp64"):

@@ -216,7 +216,7 @@ extern "C" hg_status hg_batch_create(int32_t n_grids, const hg_grid *const *grid
     b->n_grids = n_grids;
     b->total = ray_begin[n_grids];
     cudaGetDevice(&b->device);
-    cudaError_t e = cudaMalloc(&b->d_entries, ent.size() * sizeof(BatchEntry));
+    cudaError_t e = device_malloc((void **)&b->d_entries, ent.size() * sizeof(BatchEntry));
     if (e == cudaSuccess) e = cudaMemcpy(b->d_entries, ent.data(), ent.size() * sizeof(BatchEntry), cudaMemcpyHostToDevice);
     for (int f = 0; f < 2 && e == cudaSuccess; f++) {
         hg_batch::Queue &Q = b->q[f];
@@ -235,9 +235,9 @@ extern "C" hg_status hg_batch_create(int32_t n_grids, const hg_grid *const *grid
         Q.n_grids = (int)perm.size();
         Q.nav = f == 1 ? 3 : (n_ropes == 0 ? 0 : (n_ropes == Q.n_grids ? 1 : 2));
         Q.total = qbeg.back();
-        e = cudaMalloc(&Q.d_qbeg, qbeg.size() * sizeof(int64_t));
-        if (e == cudaSuccess) e = cudaMalloc(&Q.d_perm, perm.size() * sizeof(int32_t));
-        if (e == cudaSuccess) e = cudaMalloc(&Q.d_counter, sizeof(unsigned long long));
+        e = device_malloc((void **)&Q.d_qbeg, qbeg.size() * sizeof(int64_t));
+        if (e == cudaSuccess) e = device_malloc((void **)&Q.d_perm, perm.size() * sizeof(int32_t));
+        if (e == cudaSuccess) e = device_malloc((void **)&Q.d_counter, sizeof(unsigned long long));
         if (e == cudaSuccess) e = cudaMemcpy(Q.d_qbeg, qbeg.data(), qbeg.size() * sizeof(int64_t), cudaMemcpyHostToDevice);
         if (e == cudaSuccess) e = cudaMemcpy(Q.d_perm, perm.data(), perm.size() * sizeof(int32_t), cudaMemcpyHostToDevice);
     }
@@ -340,11 +340,11 @@ extern "C" hg_status hg_autotune(hg_grid *g, int64_t n, const double *o, const d
         return HG_EINVAL;
     }
     cudaStream_t s = (cudaStream_t)stream;
-    void *tau = nullptr;
-    int32_t *nc = nullptr;
-    cudaError_t e = cudaMallocAsync(&tau, (size_t)n * 8, s);
-    if (e == cudaSuccess) e = cudaMallocAsync((void **)&nc, (size_t)n * 4, s);
+    Scratch scratch;
+    cudaError_t e = scratch_get(scratch, (size_t)n * 12, s);
     if (e != cudaSuccess) return cuda_err(e, "hg_autotune scratch");
+    void *tau = scratch.p;
+    int32_t *nc = reinterpret_cast<int32_t *>(static_cast<unsigned char *>(scratch.p) + (size_t)n * 8);
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
@@ -387,8 +387,7 @@ extern "C" hg_status hg_autotune(hg_grid *g, int64_t n, const double *o, const d
                 }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    cudaFreeAsync(tau, s);
-    cudaFreeAsync(nc, s);
+    scratch_put(scratch, s);
     cudaStreamSynchronize(s);
     if (st != HG_OK) return st;
     TuneEntry &T = g->tuned[precision];

@@ -15,6 +15,7 @@
 #include <algorithm>
 
 #include "hg_internal.h"
+#include "scratch.h"
 #include "gbuild.h"
 #include "model_eval.h"
 
@@ -34,7 +35,7 @@ __global__ void __launch_bounds__(256) build_eval_kernel(const ModelView M, cons
 }
 
 static cudaError_t upload(void **dst, const void *src, size_t bytes, cudaStream_t s) {
-    cudaError_t e = cudaMalloc(dst, std::max<size_t>(bytes, 16));
+    cudaError_t e = device_malloc(dst, std::max<size_t>(bytes, 16));
     if (e == cudaSuccess && bytes) e = cudaMemcpyAsync(*dst, src, bytes, cudaMemcpyHostToDevice, s);
     return e;
 }
@@ -170,9 +171,9 @@ static hg_status device_neighbors(const NbrTree &T, int64_t nl, cudaStream_t s, 
     uint32_t err = 0;
     const int64_t nw = 6 * nl;
     const unsigned blocks = (unsigned)std::max<int64_t>(1, std::min<int64_t>((nw + 255) / 256, (int64_t)sm_count() * 16));
-    cudaError_t e = cudaMalloc((void **)&d_cnt, (size_t)std::max<int64_t>(nw, 1) * sizeof(int32_t));
-    if (e == cudaSuccess) e = cudaMalloc((void **)&d_off, (size_t)(nw + 1) * sizeof(int64_t));
-    if (e == cudaSuccess) e = cudaMalloc((void **)&d_err, sizeof(uint32_t));
+    cudaError_t e = device_malloc((void **)&d_cnt, (size_t)std::max<int64_t>(nw, 1) * sizeof(int32_t));
+    if (e == cudaSuccess) e = device_malloc((void **)&d_off, (size_t)(nw + 1) * sizeof(int64_t));
+    if (e == cudaSuccess) e = device_malloc((void **)&d_err, sizeof(uint32_t));
     if (e == cudaSuccess) e = cudaMemsetAsync(d_err, 0, sizeof(uint32_t), s);
     if (e == cudaSuccess && nw > 0) {
         nbr_count_kernel<<<blocks, 256, 0, s>>>(T, nl, d_cnt, d_err);
@@ -186,8 +187,8 @@ static hg_status device_neighbors(const NbrTree &T, int64_t nl, cudaStream_t s, 
     if (hs == HG_OK) {
         e = cudaMemcpyAsync(&total, d_off + nw, sizeof(int64_t), cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-        if (e == cudaSuccess) e = cudaMalloc((void **)&d_ids, (size_t)std::max<int64_t>(total, 1) * sizeof(int32_t));
-        if (e == cudaSuccess) e = cudaMalloc((void **)&d_area, (size_t)std::max<int64_t>(total, 1) * sizeof(int64_t));
+        if (e == cudaSuccess) e = device_malloc((void **)&d_ids, (size_t)std::max<int64_t>(total, 1) * sizeof(int32_t));
+        if (e == cudaSuccess) e = device_malloc((void **)&d_area, (size_t)std::max<int64_t>(total, 1) * sizeof(int64_t));
         if (e == cudaSuccess && nw > 0) {
             nbr_fill_kernel<<<blocks, 256, 0, s>>>(T, nl, d_off, d_ids, d_area, d_err);
             note_launches(1);
@@ -307,7 +308,7 @@ struct BuildBufs {
     template <class T>
     cudaError_t alloc(T **p, int64_t count) {
         *p = nullptr;
-        cudaError_t e = cudaMalloc((void **)p, (size_t)std::max<int64_t>(count, 1) * sizeof(T));
+        cudaError_t e = device_malloc((void **)p, (size_t)std::max<int64_t>(count, 1) * sizeof(T));
         if (e == cudaSuccess) ptrs.push_back(*p);
         return e;
     }

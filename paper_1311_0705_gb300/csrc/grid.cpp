@@ -614,7 +614,7 @@ hg_status load_grid_impl(const hg_grid_desc *desc, const int32_t *ropes, int32_t
         if (e != cudaSuccess) return cuda_fail(e, "hg_load_grid: no CUDA device");
         g->device = dev;
         auto upload = [&](void **dst, const void *src, size_t bytes) -> cudaError_t {
-            cudaError_t r = cudaMalloc(dst, bytes);
+            cudaError_t r = hg::device_malloc(dst, bytes);
             if (r != cudaSuccess) return r;
             return cudaMemcpy(*dst, src, bytes, cudaMemcpyHostToDevice);
         };

@@ -667,7 +667,7 @@ extern "C" hg_status hg_load_model(const hg_model *model, hg_dmodel **out) {
     }
     const size_t per = (model->kind == HG_MODEL_TORUS) ? 5 : 1;
     const size_t bytes = std::max<size_t>(8, (size_t)model->n_table * per * sizeof(double));
-    cudaError_t e = cudaMalloc(&dm->d_table, bytes);
+    cudaError_t e = device_malloc(&dm->d_table, bytes);
     if (e == cudaSuccess && model->n_table > 0)
         e = cudaMemcpy(dm->d_table, model->table, (size_t)model->n_table * per * sizeof(double),
                        cudaMemcpyHostToDevice);

@@ -13,9 +13,12 @@
 //     that a new stream that got a destroyed one's handle is ordered too.
 //   * Under stream capture blocks come from and go to the allocator, as graph nodes: a graph's scratch is its own.
 //   * The list of kept blocks is a fixed array: nothing here allocates on the host or throws.
-//   * When an allocation fails the kept blocks are released and it is tried again.
+//   * When an allocation of this library fails the kept blocks are released and it is tried again; for other
+//     allocators of the program there is hg_release_scratch.
 // (Kept blocks are freed by cudaFreeAsync throughout: after cudaFree the pool went on counting them as used.)
 #include "scratch.h"
+
+#include "hg_internal.h"
 
 #include <cstdint>
 #include <mutex>
@@ -85,11 +88,38 @@ Blocks take_all(Device &d) {
     return out;
 }
 
-// Free a block once its last use has ended, in `stream`'s order.
+// Free a block in the order of `stream`, whose own it was or whose work has ended.
 void release_in(const Scratch &s, cudaStream_t stream) {
     cudaStreamWaitEvent(stream, s.done, 0);
     cudaFreeAsync(s.p, stream);
     cudaEventDestroy(s.done);
+}
+
+// Free a device's kept blocks once their last uses have ended (the host waits), and have the pool give their memory back to
+// the system, on a stream of its own; false when there were none.
+bool release_kept(int device) {
+    Blocks all;
+    {
+        std::lock_guard<std::mutex> lock(g_mtx);
+        all = take_all(g_dev[device]);
+    }
+    if (all.n == 0) return false;
+    int cur = 0;
+    cudaGetDevice(&cur);
+    if (cur != device) cudaSetDevice(device);
+    {
+        const RelaxedCapture relaxed;
+        cudaStream_t stream = nullptr;
+        if (!ok(cudaStreamCreateWithFlags(&stream, cudaStreamNonBlocking))) stream = nullptr;
+        for (int i = 0; i < all.n; i++) {
+            ok(cudaEventSynchronize(all.v[i].s.done));
+            release_in(all.v[i].s, stream);
+        }
+        ok(cudaStreamSynchronize(stream));
+        if (stream) cudaStreamDestroy(stream);
+    }
+    if (cur != device) cudaSetDevice(cur);
+    return true;
 }
 
 }  // namespace
@@ -130,17 +160,7 @@ cudaError_t scratch_get(Scratch &s, size_t bytes, cudaStream_t stream) {
     e = cudaMallocAsync(&s.p, bytes, stream);
     if (e == cudaErrorMemoryAllocation) {
         cudaGetLastError();
-        Blocks all;
-        {
-            std::lock_guard<std::mutex> lock(g_mtx);
-            all = take_all(g_dev[device]);
-        }
-        for (int i = 0; i < all.n; i++) release_in(all.v[i].s, stream);
-        if (all.n > 0) {
-            const RelaxedCapture relaxed;
-            cudaStreamSynchronize(stream);
-        }
-        e = cudaMallocAsync(&s.p, bytes, stream);
+        if (release_kept(device)) e = cudaMallocAsync(&s.p, bytes, stream);
     }
     if (!ok(e)) {
         s = Scratch();
@@ -189,23 +209,35 @@ void scratch_put(Scratch &s, cudaStream_t stream) {
 
 void scratch_users(int device, int delta) {
     if (device < 0 || device >= kDevices) return;
-    Blocks all;
+    bool last;
     {
         std::lock_guard<std::mutex> lock(g_mtx);
         g_dev[device].users += delta;
-        if (g_dev[device].users <= 0) all = take_all(g_dev[device]);
+        last = g_dev[device].users <= 0;
     }
-    if (all.n == 0) return;
-    int cur = 0;
-    cudaGetDevice(&cur);
-    if (cur != device) cudaSetDevice(device);
-    const RelaxedCapture relaxed;
-    for (int i = 0; i < all.n; i++) {
-        cudaEventSynchronize(all.v[i].s.done);
-        cudaFreeAsync(all.v[i].s.p, 0);
-        cudaEventDestroy(all.v[i].s.done);
+    if (last) release_kept(device);
+}
+
+cudaError_t device_malloc(void **p, size_t bytes) {
+    cudaError_t e = cudaMalloc(p, bytes);
+    int device = -1;
+    if (e == cudaErrorMemoryAllocation && cudaGetDevice(&device) == cudaSuccess && device < kDevices) {
+        cudaGetLastError();
+        if (release_kept(device)) e = cudaMalloc(p, bytes);
     }
-    if (cur != device) cudaSetDevice(cur);
+    ok(e);
+    return e;
 }
 
 }  // namespace hg
+
+extern "C" hg_status hg_release_scratch(void) {
+    int device = -1;
+    const cudaError_t e = cudaGetDevice(&device);
+    if (!hg::ok(e)) {
+        hg::set_error("hg_release_scratch: %s", cudaGetErrorString(e));
+        return HG_ECUDA;
+    }
+    if (device < hg::kDevices) hg::release_kept(device);
+    return HG_OK;
+}

@@ -21,5 +21,7 @@ void scratch_put(Scratch &s, cudaStream_t stream);
 // A grid or ray plan of a device came to life (+1) or was released (-1); with the last one the kept blocks
 // are released.
 void scratch_users(int device, int delta);
+// cudaMalloc on the current device; when it fails, once more without the kept blocks.
+cudaError_t device_malloc(void **p, size_t bytes);
 
 }  // namespace hg

@@ -19,7 +19,7 @@ struct Event { cudaStream_t stream = nullptr; long at = -1; };
 std::map<void *, size_t> live;
 std::map<cudaStream_t, long> sent, done;
 size_t used = 0, limit = (size_t)1 << 40;
-int cross = 0, host_waits = 0, unsafe = 0;
+int cross = 0, unsafe = 0;
 cudaStream_t capture = nullptr;
 cudaError_t last = cudaSuccess;
 cudaStreamCaptureMode mode = cudaStreamCaptureModeGlobal;
@@ -41,6 +41,7 @@ extern "C" {
 cudaError_t cudaGetDevice(int *d) { *d = 0; return cudaSuccess; }
 cudaError_t cudaSetDevice(int) { return cudaSuccess; }
 cudaError_t cudaGetLastError() { cudaError_t e = last; last = cudaSuccess; return e; }
+const char *cudaGetErrorString(cudaError_t) { return "error"; }
 cudaError_t cudaMalloc(void **p, size_t n) { return take(p, n); }
 cudaError_t cudaMallocAsync(void **p, size_t n, cudaStream_t) { return take(p, n); }
 cudaError_t cudaFreeAsync(void *p, cudaStream_t) { give(p); return cudaSuccess; }
@@ -54,7 +55,12 @@ cudaError_t cudaEventDestroy(cudaEvent_t e) { delete (Event *)e; return cudaSucc
 cudaError_t cudaEventRecord(cudaEvent_t e, cudaStream_t s) { auto v = (Event *)e; v->stream = s; v->at = sent[s]; return cudaSuccess; }
 static void check_mode() { if (mode != cudaStreamCaptureModeRelaxed) unsafe++; }
 cudaError_t cudaEventQuery(cudaEvent_t e) { check_mode(); return complete((Event *)e) ? cudaSuccess : fail(cudaErrorNotReady); }
-cudaError_t cudaEventSynchronize(cudaEvent_t e) { check_mode(); host_waits += !complete((Event *)e); return cudaSuccess; }
+cudaError_t cudaEventSynchronize(cudaEvent_t e) {
+    auto v = (Event *)e;
+    check_mode();
+    if (!complete(v)) done[v->stream] = v->at;
+    return cudaSuccess;
+}
 cudaError_t cudaStreamWaitEvent(cudaStream_t s, cudaEvent_t e, unsigned) {
     auto v = (Event *)e;
     cross += v->stream != s && !complete(v);
@@ -76,13 +82,14 @@ void t_put(void *v, long s) { hg::scratch_put(*(hg::Scratch *)v, (cudaStream_t)s
 void t_users(int delta) { hg::scratch_users(0, delta); }
 void t_rest(long s) { done[(cudaStream_t)s] = sent[(cudaStream_t)s]; }
 void t_capture(long s) { capture = (cudaStream_t)s; }
+void t_forget() { used = 0; live.clear(); }
 void t_limit(size_t n) { limit = n; }
 size_t t_used() { return used; }
 int t_blocks() { return (int)live.size(); }
 int t_cross() { return cross; }
-int t_host_waits() { return host_waits; }
 int t_unsafe() { return unsafe; }
 long t_last() { return last; }
+long t_malloc(size_t n) { void *p; return hg::device_malloc(&p, n); }
 size_t t_address(void *v) { return (size_t)((hg::Scratch *)v)->p; }
 }
 """
@@ -98,6 +105,7 @@ class Fake:
         lib.t_last.restype = lib.t_get.restype = ctypes.c_long
         lib.t_put.argtypes = [ctypes.c_void_p, ctypes.c_long]
         lib.t_address.argtypes = [ctypes.c_void_p]
+        lib.t_malloc.argtypes, lib.t_malloc.restype = [ctypes.c_size_t], ctypes.c_long
         lib.t_limit.argtypes = [ctypes.c_size_t]
         lib.t_get.argtypes = [ctypes.c_size_t, ctypes.c_long, ctypes.POINTER(ctypes.c_void_p)]
 
@@ -124,7 +132,8 @@ def fake(tmp_path):
     (tmp_path / "runtime.cpp").write_text(RUNTIME)
     so = str(tmp_path / "scratch.so")
     subprocess.run(["g++", "-O1", "-std=c++17", "-shared", "-fPIC", "-I", os.path.join(cuda, "include"), "-I", CSRC, "-I",
-                    os.path.join(ROOT, "include"), str(tmp_path / "runtime.cpp"), os.path.join(CSRC, "scratch.cpp"), "-o", so], check=True)
+                    os.path.join(ROOT, "include"), str(tmp_path / "runtime.cpp"), os.path.join(CSRC, "scratch.cpp"), os.path.join(CSRC, "common.cpp"),
+                    "-o", so], check=True)
     f = Fake(ctypes.CDLL(so))
     f.lib.t_users(1)
     yield f
@@ -189,6 +198,24 @@ def test_allocations_that_fail_are_tried_again_without_the_kept_blocks(fake):
     assert fake.reused(800 * MB, 2)
     e, _ = fake.get(2000 * MB, 2)
     assert e == 2  # cudaErrorMemoryAllocation
+
+
+def test_grids_and_models_get_the_kept_memory(fake):
+    fake.call(900 * MB, 1)
+    fake.lib.t_limit(1000 * MB)
+    assert fake.lib.t_malloc(800 * MB) == 0 and fake.lib.t_used() == 800 * MB
+    assert fake.lib.t_malloc(800 * MB) == 2 and fake.lib.t_last() == 0
+    fake.lib.t_forget()
+
+
+def test_kept_blocks_are_given_back_on_request(fake):
+    for s in (1, 2, 3):
+        fake.call(500 * MB, s)
+    e, held = fake.get(400 * MB, 2)  # in use: not given back
+    assert fake.lib.hg_release_scratch() == 0
+    assert fake.lib.t_used() == 500 * MB
+    fake.lib.t_put(held, 2)
+    assert fake.reused(500 * MB, 2)  # kept as before
 
 
 def test_no_error_is_left_behind(fake):

@@ -54,3 +54,25 @@ def test_every_turn_ends_with_the_results_of_single_calls(hg):
     [t.start() for t in threads]
     [t.join() for t in threads]
     assert not errors and turns == [30] * len(turns)
+
+
+def test_kept_scratch_is_given_back_on_request(hg):
+    grid = _grid(hg)
+    o, k = (torch.tensor(a, device="cuda") for a in synth.emission_rays(9, 400_000))
+
+    def step():
+        R = hg.prepare_rays(grid, o, k)
+        out = R.trace_stage()
+        R.free()
+        torch.cuda.synchronize()
+        return out
+
+    first = step()
+    kept = torch.cuda.mem_get_info()[0]
+    hg.release_scratch()
+    freed = torch.cuda.mem_get_info()[0] - kept
+    assert freed > 300 << 20, freed  # 64 staged entries of 16 bytes per ray and more
+    hg.release_scratch()  # nothing left: fine
+    again = step()
+    assert torch.equal(again[1], first[1])
+    torch.testing.assert_close(again[0], first[0], rtol=1e-12, atol=0)
