@@ -131,7 +131,7 @@ def fake(tmp_path):
     cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
     (tmp_path / "runtime.cpp").write_text(RUNTIME)
     so = str(tmp_path / "scratch.so")
-    subprocess.run(["g++", "-O1", "-std=c++17", "-shared", "-fPIC", "-I", os.path.join(cuda, "include"), "-I", CSRC, "-I",
+    subprocess.run(["g++", "-O1", "-std=c++17", "-shared", "-fPIC", "-Wl,-Bsymbolic", "-I", os.path.join(cuda, "include"), "-I", CSRC, "-I",
                     os.path.join(ROOT, "include"), str(tmp_path / "runtime.cpp"), os.path.join(CSRC, "scratch.cpp"), os.path.join(CSRC, "common.cpp"),
                     "-o", so], check=True)
     f = Fake(ctypes.CDLL(so))
