@@ -7,6 +7,7 @@
 #include <atomic>
 #include <system_error>
 #include <memory>
+#include <new>
 #include <thread>
 #include <vector>
 
@@ -399,7 +400,11 @@ hg_status load_grid_impl(const hg_grid_desc *desc, const int32_t *ropes, int32_t
         }
     }
     const int64_t n = D.n_nodes, nl = D.n_leaves;
-    std::unique_ptr<hg_grid> g(new hg_grid());
+    std::unique_ptr<hg_grid> g(new (std::nothrow) hg_grid());
+    if (!g) {
+        hg::set_error("hg_load_grid: out of host memory");
+        return HG_ENOMEM;
+    }
     try {
         // node depths for the descent limit
         std::vector<int32_t> depth((size_t)n, 0);
@@ -530,7 +535,7 @@ hg_status load_grid_impl(const hg_grid_desc *desc, const int32_t *ropes, int32_t
             try {
                 const int threads = (int)std::min<int64_t>(std::max(1u, std::thread::hardware_concurrency()), nl / chunk);
                 for (int t = 1; t < threads; t++) pool.emplace_back(fill);
-            } catch (const std::system_error &) {  // fewer threads, then
+            } catch (const std::exception &) {  // no thread or no memory for one: fewer threads, then
             }
             fill();
             for (auto &th : pool) th.join();
