@@ -559,8 +559,9 @@ hg_status hg_batch_trace(hg_batch *b, const double *o, const double *d, const do
 hg_status hg_release_scratch(void);
 
 /* ------------------------------------------------------------------------ autotuner
- * Time candidate launch configurations (threads per block, shared-memory
- * tree nodes, schedule) on a sample of n rays with CUDA events, keep the
+ * Time candidate launch configurations (threads per block, schedule and, for
+ * 96-byte records, shared-memory tree nodes and min_blocks: 64-byte ones
+ * report the defaults) on a sample of n rays with CUDA events, keep the
  * fastest for this grid and precision (used when opts fields are 0 / -1),
  * and return it in *best.  Synchronises the stream. */
 hg_status hg_autotune(hg_grid *g, int64_t n, const double *o, const double *d, int32_t precision,

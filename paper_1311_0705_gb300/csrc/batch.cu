@@ -350,18 +350,22 @@ extern "C" hg_status hg_autotune(hg_grid *g, int64_t n, const double *o, const d
     cudaEventCreate(&e1);
     const int node_bytes = node_bytes_of(g->d);
     const int blocks[] = {128, 256};
-    const int smem_kb[] = {0, 8, 32, 64};
+    // walks of 64-byte records stage no nodes and have one form each: neither choice makes a difference there, and
+    // the defaults stand for both
+    const bool one_form = g->d.recf != nullptr;
+    const int nodes_at[] = {one_form ? kWalkNodes : 0, 8 * 1024 / node_bytes, 32 * 1024 / node_bytes, 64 * 1024 / node_bytes};
+    const int n_nodes_at = one_form ? 1 : 4;
     hg_trace_opts win{};
     float win_ms = 1e30f;
     hg_status st = HG_OK;
     for (int sched = 1; sched <= 3 && st == HG_OK; sched++)
-        for (int occ = 3; occ <= 4; occ++)
+        for (int occ = one_form ? 4 : 3; occ <= 4; occ++)
             for (int bl : blocks)
-                for (int kb : smem_kb) {
+                for (int j = 0; j < n_nodes_at; j++) {
                     hg_trace_opts op{};
                     op.precision = precision;
                     op.block = bl;
-                    op.smem_nodes = (int)std::min<int64_t>(g->d.n_nodes, (int64_t)kb * 1024 / node_bytes);
+                    op.smem_nodes = (int)std::min<int64_t>(g->d.n_nodes, nodes_at[j]);
                     op.schedule = sched;
                     op.min_blocks = occ;
                     st = hg_trace_rays(g, n, o, d, nullptr, 1.0, &op, tau, nc, nullptr, stream);

@@ -524,7 +524,6 @@ int sm_count() {
 // (setup_nodes): its deep levels come through L1 as well, and with 32 KB of
 // nodes (and the 16 KB work lattice) per block the k-d preparation of 1e6
 // rays took 0.52 ms against 0.29 ms.
-constexpr int kWalkNodes = 64;
 int setup_nodes(const hg_grid *g) {
     const int node_bytes = node_bytes_of(g->d);
     return (int)std::min<int64_t>(g->d.n_nodes, (8 * 1024) / node_bytes);

@@ -212,6 +212,8 @@ __device__ __forceinline__ void walk_io(const TraceArgs &A, WalkIO &io) {
     io.int_t = A.int_t;
 }
 
+constexpr int kWalkNodes = 64;  // top tree nodes that the walks of 96-byte records stage by default (trace.cu)
+
 typedef void (*KernelFn)(const TraceArgs);
 KernelFn pick_kernel_f(int mode, int prec);  // single-precision records (tracef.cu)
 

@@ -41,3 +41,21 @@ def test_small_batches_of_a_tuned_grid(hg, kind):
     n = hg.launch_count()
     hg.trace_rays(grid, o, k, schedule=3)
     assert hg.launch_count() - n == plain + 1
+
+
+def test_only_what_makes_a_difference_is_tried(hg):
+    model = synth.make_disk()
+    o, k = (torch.tensor(a, device="cuda") for a in synth.emission_rays(4, 500))
+    o *= 0.3
+    for half, shapes in ((1.0, 3 * 2), (0.3, 3 * 2 * 2 * 4)):  # 64-byte records: schedules, blocks; 96-byte: all
+        model = synth.make_disk(half=half)
+        grid = hg.load_grid(hg.build_grid(model, synth.BuildParams(kind=0, delta_max=1e-3, max_level=8, seed=3)))
+        n = hg.launch_count()
+        for s in (1, 2, 3):
+            hg.trace_rays(grid, o, k, schedule=s)
+        once = (hg.launch_count() - n) / 3
+        n = hg.launch_count()
+        cfg, _ = hg.autotune(grid, o, k)
+        assert hg.launch_count() - n == 4 * shapes * once  # one untimed and three timed calls each
+        if half == 1.0:
+            assert (cfg["smem_nodes"], cfg["min_blocks"]) == (64, 4)
