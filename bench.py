@@ -55,13 +55,18 @@ L2_FLUSH_BYTES = 512 << 20
 # what bounds the walk besides the copy bandwidth: random gathers of 64-byte records from a 2 GB array
 # sustained 19.6 G records/s (1.25 TB/s) in a separate probe (96-byte records 13.2 G/s, 1.27 TB/s), and FP64
 # add / fused multiply-add issued 16.5 G warp instructions/s (0.053 per cycle per SM) whether 32, 16 or 1
-# lane was active, i.e. 528 G lane operations/s at full warps; per crossing the walk of grids with
-# single-precision bounds (all of these workloads) issues 4 FP64 instructions (2 for the time of the wall
-# that is crossed, ds, the fused sum; under FP32-Kahan the sum leaves the FP64 pipe and the FP32 cast of ds
-# joins it), the walk of other grids 10
-RANDOM_GATHER_GBS = 1.25e3
+# lane was active, i.e. 528 G lane operations/s at full warps; per crossing the walk of 64-byte records issues
+# 4 FP64 instructions (2 for the time of the wall that is crossed, ds, the fused sum; under FP32-Kahan the sum
+# leaves the FP64 pipe and the FP32 cast of ds joins it), the walk of 96-byte records 10
+RANDOM_GATHER_GBS = {64: 1.25e3, 96: 1.27e3}
 FP64_OPS_PER_S = 528e9
-FP64_OPS_PER_CROSSING = {"fp64": 4, "fp32k": 4}
+FP64_OPS_PER_CROSSING = {64: 4, 96: 10}
+
+
+def record_bytes(grid, host) -> int:
+    """Bytes of the leaf records a loaded grid got (64 where its bounds are single-precision numbers): 64-byte ones and
+    their nodes (8 bytes each, 2 per leaf; octrees 16, 8/7 per leaf) stay below 96 per leaf beside the work lattice."""
+    return 96 if grid.device_bytes - 4 * 16 ** 3 >= 96 * host.n_leaves else 64
 
 
 # ----------------------------------------------------------------------------- distributed plumbing
@@ -472,7 +477,8 @@ def run_ours(args):
     traffic = recorded_traffic(args.workload, prec)
     tot_cross = sum(int(g["nc"].sum().item()) for g in grids)
     byte_per_cross = tot_bytes / max(1, tot_cross)
-    fp64_gcross = FP64_OPS_PER_S / FP64_OPS_PER_CROSSING[prec]
+    rec = max(record_bytes(g["grid"], g["host"]) for g in grids)
+    fp64_gcross = FP64_OPS_PER_S / FP64_OPS_PER_CROSSING[rec]
     roofline = dict(bound="hbm", achieved=round(achieved, 1), peak=peak, unit="GB/s", frac=round(achieved / peak, 4),
                     traffic=traffic, kernel="trace_kernel, one walk for optical depth and staged emission over "
                                             "prepared rays (hg_rays_trace_stage)",
@@ -481,12 +487,12 @@ def run_ours(args):
                         achieved_gcross_per_s=round(tot_cross / tot_time / 1e6, 2),
                         fp64_issue_gcross_per_s=round(fp64_gcross / 1e9, 1),
                         fp64_issue_frac_of_peak=round(fp64_gcross * byte_per_cross / 1e9 / peak, 3),
-                        random_gather_gbs=RANDOM_GATHER_GBS,
-                        random_gather_frac_of_peak=round(RANDOM_GATHER_GBS / peak, 3),
-                        note=f"{FP64_OPS_PER_CROSSING[prec]} FP64 instructions per crossing at the 528 G lane "
+                        random_gather_gbs=RANDOM_GATHER_GBS[rec],
+                        random_gather_frac_of_peak=round(RANDOM_GATHER_GBS[rec] / peak, 3),
+                        note=f"{FP64_OPS_PER_CROSSING[rec]} FP64 instructions per crossing at the 528 G lane "
                              "operations/s this GPU issues with full warps bound the walk at fp64_issue_gcross_per_s, "
                              "i.e. fp64_issue_frac_of_peak "
-                             "of the copy bandwidth in algorithmic bytes; random 64-byte record gathers from "
+                             f"of the copy bandwidth in algorithmic bytes; random {rec}-byte record gathers from "
                              "beyond L2 sustain random_gather_gbs (separate probes); L2 serves part of the records"))
 
     # the emitted cell sequences of the last step, on the host (the navigation comparison reads a sample)

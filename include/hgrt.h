@@ -319,8 +319,8 @@ typedef struct hg_trace_opts {
                             than 64 registers); 3 or 4 resident 256-thread blocks per SM the register
                             budget of the walks of 96-byte records is cut for (80 or 64 registers; each walking
                             thread also keeps its ray's origin, direction and 1/d in 72 bytes of shared
-                            memory).  Walks of 64-byte records have one form of 64 registers (accepted and
-                            checked, then ignored) */
+                            memory).  Walks of 64-byte records have one form each, of 64 registers (80 for
+                            hg_find_interactions): accepted and checked, then ignored */
     int32_t split;       /* HG_SPLIT_AUTO (0), HG_SPLIT_OFF or HG_SPLIT_FORCE; see below */
     int64_t max_steps;   /* per-ray step limit; 0 = 4 * n_leaves + 64 */
 } hg_trace_opts;

@@ -604,7 +604,8 @@ void set_smem_limits() {
 }
 
 // The walking kernel for a grid.  Grids with single-precision records have one variant per mode (either
-// tree and navigation, 64 registers): their tree descents are rare and read the node format at run time.
+// tree and navigation; 64 registers, the interaction search 80): their tree descents are rare and read the node format
+// at run time.
 KernelFn walk_kernel(const hg_grid *g, int mode, int prec, int occ) {
     return g->d.recf ? pick_kernel_f(mode, prec) : pick_kernel(g->d.kind, mode, prec, occ, g->d.nav);
 }
@@ -1334,8 +1335,9 @@ extern "C" hg_status hg_find_interactions(const hg_grid *g, int64_t n, const dou
     int prec, block, smem_nodes, schedule, min_blocks, split;
     int64_t max_steps;
     if ((st = resolve_opts(g, opts, prec, block, smem_nodes, schedule, min_blocks, max_steps, split)) != HG_OK) return st;
-    // The search keeps the drawn depth and the interaction state beside the walk's own: cut to 64
-    // registers it spills, and at 80 (3 blocks/SM) it runs about a tenth faster on the disk grids.
+    // The search keeps the drawn depth and the interaction state beside the walk's own: on 96-byte records, cut to 64
+    // registers it spills, and at 80 (3 blocks/SM) it runs about a tenth faster on the disk grids.  (The search of 64-byte
+    // records is compiled for 80, trace_kernel_f.)
     if (!(opts && opts->min_blocks > 0)) min_blocks = 3;
     TraceArgs A{};
     A.G = g->d;

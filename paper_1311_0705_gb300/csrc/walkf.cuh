@@ -61,15 +61,14 @@
 // kRefill of a warp are idle and are refilled together from queue items taken 32
 // at a time.
 //
-// Measured, 1e6 rays on the disk octree, FP64 optical depth: the walk of walk.cuh 969 us; these records
-// and decisions inside its loop 960 us (the refill -- queue atomic, order, start record, first leaf -- and
-// the searches are chains of dependent loads that every round of a warp waits for: issue slots 38 % used,
-// 16 of 32 lanes active); with the lane states 598 us (59 %, 20 lanes; L1 wavefronts 57-62 %).  DRAM reads
-// 2.3 -> 1.1 GB.  FP64 pipe 46 % busy: its 4 operations per crossing bound the walk at 235 us.  What is left is
-// instructions, so they are few: the steps to equal neighbors in the spare bits of the wall slot, one comparison of
-// the high words for "later than now, before the end" (the rest in the branch not taken), the two parts of eps in
-// shared memory, and no register spills in the optical-depth walk (20 bytes of them cost it 12 %): calls
-// 905 -> 797 us (1e6 rays, disk octree), 12.88 -> 11.57 ms (1e7, torus, FP32K).
+// Measured, 1e6 rays on the disk octree, FP64 optical depth: walk 969 us with walk.cuh, 527 us here; calls 1248 -> 697 us, and
+// 18.6 -> 11.4 ms for 1e7 rays through the torus (FP32K).  The records and decisions alone, inside the loop of walk.cuh, gained
+// nothing (960 us): every round of a warp waited there for its lanes' chains of dependent refill loads (queue atomic,
+// order, start record, first leaf) and list searches, which the lane states put under way together.  The four FP64
+// operations per crossing bound the walk at 235 us; what it lives on is instructions, so they are few: the steps to equal
+// neighbors in the spare bits of the wall slot, one comparison of the high words for "later than now, before the end" (the rest in
+// the branch not taken), the two parts of eps in shared memory, and no register spills in the optical-depth walk (20 bytes
+// of them cost it 12 %).
 #pragma once
 
 #include "walk.cuh"
@@ -372,8 +371,8 @@ __device__ __forceinline__ bool locate_step(const DevGrid &G, const WalkIO &io, 
 // queue is empty.
 enum { LANE_WALK = 0, LANE_START = 1, LANE_NODE = 2, LANE_DONE = 3, LANE_EXIT = 4 };
 // Idle lanes of a warp that are refilled together: a refill is ~100 instructions whatever the number of
-// lanes taking part, an idle lane costs its share of a round.  2, 4, 6, 8 lanes: disk octree (1e6 rays) 887,
-// 873, 867, 858 us, torus (1e7) 11.62, 11.48, 11.67, 11.90 ms per call.
+// lanes taking part, an idle lane costs its share of a round.  2, 4, 5, 6, 8 lanes: disk octree (1e6 rays) 741, 715, 708, 703,
+// 693 us, torus (1e7) 11.57, 11.32, 11.37, 11.47, 11.66 ms per call.
 constexpr int kRefill = 5;
 struct PoolItem {
     int64_t item;  // queue item: a ray, or n_rays + s for path segment s
