@@ -162,9 +162,10 @@ __device__ __forceinline__ RayStartF start_f(const RayStart &R, const double *__
     for (int a = 0; a < 3; a++) {
         const double x = o[3 * r + a], k = d[3 * r + a];
         S.o[a] = dzero(x) ? 0.0 : x;
-        const float m = fabsf(near_float(k)), mo = fabsf(near_float(x));
-        exact = exact || !(dzero(x) || (mo >= 0x1p-60f && mo <= 0x1p20f)) ||
-                !(dzero(k) || (m >= 0x1p-30f && m <= 0x1p30f));
+        // zero, or of magnitude [2^-60, 2^20) (origin), [2^-30, 2^30) (direction), on the exponents
+        const uint32_t mx = ((uint32_t)__double2hiint(x) & 0x7fffffffu) - 0x3c300000u;
+        const uint32_t mk = ((uint32_t)__double2hiint(k) & 0x7fffffffu) - 0x3e100000u;
+        exact = exact || !(dzero(x) || mx < 0x05000000u) || !(dzero(k) || mk < 0x03c00000u);
     }
     S.sg = R.sg | (exact ? SG_EXACT : 0u);
     return S;
