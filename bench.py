@@ -174,7 +174,7 @@ class ClockSampler:
 
 def kernel_source_sha() -> str:
     h = hashlib.sha256()
-    for f in ("walk.cuh", "walkf.cuh", "trace_args.cuh", "trace.cu", "tracef.cu", "hg_internal.h"):
+    for f in ("walk.cuh", "walkf.cuh", "plan_rules.h", "trace_args.cuh", "trace.cu", "tracef.cu", "hg_internal.h"):
         h.update(open(os.path.join(ROOT, "paper_1311_0705_gb300", "csrc", f), "rb").read())
     return h.hexdigest()[:16]
 
