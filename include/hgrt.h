@@ -522,7 +522,8 @@ void hg_free_model(hg_dmodel *m);
 hg_status hg_model_density(const hg_dmodel *m, int64_t n, const double *pts, double *rho, hg_stream stream);
 /* tau_t = kappa * integral_0^len rho_t(o + t d) dt by adaptive 15-point
  * Gauss-Kronrod quadrature with breakpoints at the model's kinks and edges,
- * local relative tolerance rtol.  Directions must be unit vectors. */
+ * local relative tolerance rtol.  Directions must be unit vectors.  The same
+ * call gives the same bits. */
 hg_status hg_model_tau(const hg_dmodel *m, int64_t n, const double *o, const double *d, const double *len,
                        double kappa, double rtol, double *tau, hg_stream stream);
 /* Statistics of x = a - b (dev f64[n] each): out dev f64[3] = {n, mean, population std},
